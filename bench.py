@@ -540,8 +540,8 @@ def run_ensemble(args, rank, world, local_rank):
             "speedup_vs_sequential": seq["ms_per_step"] / tun["ms_per_step"],
             "autotune": {"seconds": tune_s, "choice": list(choice) if choice else None,
                          "candidate_s": {f"{a},{b}": v for (a, b), v in cand_s.items()},
-                         "schedule": "(ilu_cta: 0 = one 8x4-row tile per warp, 1 = 2x2 tiles "
-                                     "per CTA; coarse_cluster: 0 = one CTA, 1 = cluster)",
+                         "schedule": "(ilu_cta: 0 = every tile on its own, 1 = blocks of tiles "
+                                     "per cluster; coarse_cluster: 0 = one CTA, 1 = cluster)",
                          "results_unchanged": bool(tuned_same)},
             "bitwise_equal_to_sequential": bool(same)}
 

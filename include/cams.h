@@ -249,10 +249,11 @@ int cams_set_stream(cams_handle* h, void* stream);
 
 /* Choose between the handle's equivalent kernel schedules (for an autotuner;
  * setup picks defaults):
- *   ilu_cta         ILU(0) wavefront sweeps: 0 = one 8x4-row tile per warp,
- *                   1 = 2x2 tiles per CTA with the edges inside a block in
- *                   shared memory (the same arithmetic; results are bitwise
- *                   equal); -1 = unchanged
+ *   ilu_cta         ILU(0) wavefront sweeps: 0 = every 32-row tile on its own,
+ *                   tile edges through L2, 1 = blocks of 8 tiles per
+ *                   thread-block cluster, the edges inside a block through
+ *                   distributed shared memory (the same arithmetic; results
+ *                   are bitwise equal); -1 = unchanged
  *   coarse_cluster  symmetric (MSFE) coarse solve: 0 = one CTA, 1 = across a
  *                   thread-block cluster (a different summation order); -1 =
  *                   unchanged.  The general band solve has one schedule.

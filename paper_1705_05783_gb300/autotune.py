@@ -1,7 +1,8 @@
 """Per-shape choice of the engine's equivalent kernel schedules.
 
-The ILU(0) wavefront sweeps run either one 8x4-row tile per warp or 2x2
-tiles per CTA (the same arithmetic, bitwise-equal results), and the
+The ILU(0) wavefront sweeps run either every 32-row tile on its own or
+blocks of tiles per thread-block cluster (the same arithmetic,
+bitwise-equal results), and the
 symmetric coarse solve runs in one CTA or across a thread-block cluster.
 Which is faster depends on the grid, the coarse grid and the precision, so
 `tune` times a few C-AMS iterations of a live handle under every schedule the

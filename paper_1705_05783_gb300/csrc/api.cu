@@ -59,10 +59,9 @@ struct cams_handle {
   long long launch_base = 0;
   bool single = false;          // mixed precision: FP32 preconditioner (b.f32)
   bool ilu_pipelined = true;    // false: level-scheduled sweeps (CAMS_ILU_LEVEL=1)
-  bool ilu_cta = false;         // 2 x 2 tile blocks per CTA, else one tile per warp
+  bool ilu_cta = false;         // blocks of tiles per cluster, else every tile on its own
   bool coarse_cluster = false;  // MSFE coarse solve across a cluster (CAMS_COARSE_CLUSTER=0: one CTA)
   bool coarse_inv = false;      // mixed MSFE: FP32 factor and inverse factor (CAMS_COARSE_INV=0: off)
-  int ilu_grid = 1;
   // learned surrogate of the interior basis stage (cams_set_surrogate)
   double surr_tol = 0.0;           // > 0: enabled
   int surr_b = 0, surr_n = 0, surr_chunk = 0, surr_accepted = 0;
@@ -299,7 +298,7 @@ int alloc_all(cams_handle* h) {
   if (!h->single) AL(b.P, 8 * N);
   if (h->single) {
     SingleBuffers& f = b.f32;
-    const long long S = ilu_skew_len(h->g);
+    const long long S = ilu_sweep_len(h->g, true);
     AL(f.Ad, N); AL(f.Ax, N); AL(f.Ay, N); AL(f.Az, N); AL(f.dinv, N); AL(f.d, N); AL(f.r, N);
     if (h->opt.jacobian) {
       AL(f.Axu, N); AL(f.Ayu, N); AL(f.Azu, N); AL(f.Qx, N); AL(f.Qy, N); AL(f.Qz, N);
@@ -314,12 +313,11 @@ int alloc_all(cams_handle* h) {
       AL(f.tc, coarse_ldz(h->c.Nc));
       AL(f.zpart, coarse_part_len(h->c.Nc));
     }
-    AL(f.Lx, S); AL(f.Ly, S); AL(f.Lz, S); AL(f.Ux, S); AL(f.Uy, S); AL(f.Uz, S);
-    AL(f.rds, S); AL(f.w, S); AL(f.z, S);
+    AL(f.lo, 4 * S); AL(f.up, 4 * S); AL(f.z, S);
     // slots that hold no cell must read as zero (the sweeps run branch-free over them)
-    for (float* v : {f.Lx, f.Ly, f.Lz, f.Ux, f.Uy, f.Uz, f.rds, f.w, f.z})
-      if (cudaMemset(v, 0, sizeof(float) * (size_t)S) != cudaSuccess)
-        return fail(h, CAMS_ECUDA, "cudaMemset failed");
+    if (cudaMemset(f.lo, 0, sizeof(float) * 4 * (size_t)S) != cudaSuccess ||
+        cudaMemset(f.up, 0, sizeof(float) * 4 * (size_t)S) != cudaSuccess)
+      return fail(h, CAMS_ECUDA, "cudaMemset failed");
   }
   AL(b.ent_of_cell, N);
   AL(b.ents, h->ents.size());
@@ -336,14 +334,13 @@ int alloc_all(cams_handle* h) {
   AL(b.jxt, 2LL * h->g.nx);
   AL(b.rc, h->c.Nc); AL(b.pc, h->c.Nc); AL(b.ywork, h->c.Nc);
   AL(b.dinv, N);
-  {
-    const long long S = ilu_skew_len(h->g);   // >= N
-    AL(b.Lx, S); AL(b.Ly, S); AL(b.Lz, S); AL(b.Ux, S); AL(b.Uy, S); AL(b.Uz, S);
-    AL(b.rds, S); AL(b.w, S); AL(b.z, S);
+  if (!h->single) {
+    const long long S = ilu_sweep_len(h->g, false);
+    AL(b.lo, 4 * S); AL(b.up, 4 * S); AL(b.z, S);
     // slots that hold no cell must read as zero (the sweeps run branch-free over them)
-    for (double* v : {b.Lx, b.Ly, b.Lz, b.Ux, b.Uy, b.Uz, b.rds, b.w, b.z})
-      if (cudaMemset(v, 0, sizeof(double) * (size_t)S) != cudaSuccess)
-        return fail(h, CAMS_ECUDA, "cudaMemset failed");
+    if (cudaMemset(b.lo, 0, sizeof(double) * 4 * (size_t)S) != cudaSuccess ||
+        cudaMemset(b.up, 0, sizeof(double) * 4 * (size_t)S) != cudaSuccess)
+      return fail(h, CAMS_ECUDA, "cudaMemset failed");
   }
   AL(b.ctrl, ilu_ctrl_ints(h->g));
   AL(b.r, N);
@@ -365,8 +362,7 @@ void free_all(cams_handle* h) {
   void* ptrs[] = {b.Tx, b.Ty, b.Tz, b.Tbw, b.Tbe, b.p, b.pn, b.rho, b.rhon, b.Ad, b.Ax, b.Ay,
                   b.Az, b.Cacc, b.f, b.eps, b.src, b.Abd, b.Abx, b.Aby, b.Abz, b.snap, b.P,
                   b.ent_of_cell, b.ents, b.flag, b.lscratch, b.loc, b.Acs, b.band, b.perm, b.jxt, b.rc,
-                  b.pc, b.dinv, b.r, b.rds, b.w, b.z, b.red, b.scal, b.status, b.Lx, b.Ly, b.Lz,
-                  b.Ux, b.Uy, b.Uz, b.ctrl, b.Lc, b.Lr, b.cblk, b.cdinv, b.cabort, b.fixm,
+                  b.pc, b.dinv, b.r, b.z, b.red, b.scal, b.status, b.lo, b.up, b.ctrl, b.Lc, b.Lr, b.cblk, b.cdinv, b.cabort, b.fixm,
                   b.fixc, b.fixv, b.cf, b.Qx, b.Qy, b.Qz, b.Fc, b.ywork, b.lwork,
                   // the transposed couplings are separate arrays only for a nonsymmetric A
                   b.Axu != b.Ax ? b.Axu : nullptr, b.Ayu != b.Ay ? b.Ayu : nullptr,
@@ -374,8 +370,8 @@ void free_all(cams_handle* h) {
   for (void* p : ptrs)
     if (p) cudaFree(p);
   const SingleBuffers& f = b.f32;
-  void* fptrs[] = {f.Ad, f.Ax, f.Ay, f.Az, f.dinv, f.Lx, f.Ly, f.Lz, f.Ux, f.Uy, f.Uz,
-                   f.rds, f.w, f.z, f.d, f.r, f.P, f.pc, f.Qx, f.Qy, f.Qz, f.Lc, f.Lr, f.cblk, f.cdinv,
+  void* fptrs[] = {f.Ad, f.Ax, f.Ay, f.Az, f.dinv, f.lo, f.up,
+                   f.z, f.d, f.r, f.P, f.pc, f.Qx, f.Qy, f.Qz, f.Lc, f.Lr, f.cblk, f.cdinv,
                    f.Z, f.tc, f.zpart, f.Axu != f.Ax ? f.Axu : nullptr, f.Ayu != f.Ay ? f.Ayu : nullptr,
                    f.Azu != f.Az ? f.Azu : nullptr};
   for (void* p : fptrs)
@@ -638,7 +634,7 @@ int update_operators(cams_handle* h, int force, int* n_rebuilt) {
     }
     CK(cudaEventRecord(h->ev_fork, h->stream));
     CK(cudaStreamWaitEvent(h->aux_stream, h->ev_fork, 0));
-    CK(launch_ilu_factor(h->g, b, h->ilu_pipelined, h->ilu_grid, h->ilu_cta, h->single, nonsym,
+    CK(launch_ilu_factor(h->g, b, h->ilu_pipelined, h->sms, h->single, nonsym,
                          h->aux_stream));
     CK(cudaEventRecord(h->ev_join, h->aux_stream));
   }
@@ -706,8 +702,8 @@ int update_operators(cams_handle* h, int force, int* n_rebuilt) {
   if (overlap)
     CK(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
   else
-    LAUNCH(CAMS_PROF_ILU_FACTOR, launch_ilu_factor(h->g, b, h->ilu_pipelined, h->ilu_grid,
-                                                    h->ilu_cta, h->single, nonsym, h->stream));
+    LAUNCH(CAMS_PROF_ILU_FACTOR, launch_ilu_factor(h->g, b, h->ilu_pipelined, h->sms,
+                                                    h->single, nonsym, h->stream));
   return check_status(h);
 }
 
@@ -727,8 +723,8 @@ int residual_norm(cams_handle* h, double* out) {
 int ilu_smooth(cams_handle* h) {
   const bool s = h->single;
   LAUNCH(CAMS_PROF_ILU_RESID, launch_ilu_resid(h->g, h->b, s, h->stream));
-  LAUNCH(CAMS_PROF_ILU_FWD, launch_ilu_sweep(h->g, h->b, false, h->ilu_pipelined, h->ilu_grid, h->ilu_cta, s, h->stream));
-  LAUNCH(CAMS_PROF_ILU_BWD, launch_ilu_sweep(h->g, h->b, true, h->ilu_pipelined, h->ilu_grid, h->ilu_cta, s, h->stream));
+  LAUNCH(CAMS_PROF_ILU_FWD, launch_ilu_sweep(h->g, h->b, false, h->ilu_pipelined, h->ilu_cta, s, h->stream));
+  LAUNCH(CAMS_PROF_ILU_BWD, launch_ilu_sweep(h->g, h->b, true, h->ilu_pipelined, h->ilu_cta, s, h->stream));
   LAUNCH(CAMS_PROF_ILU_APPLY, launch_ilu_apply(h->g, h->b, s, h->stream));
   return CAMS_OK;
 }
@@ -1135,14 +1131,12 @@ int cams_setup(const cams_grid* grid, const cams_fluid* fluid, const cams_option
     h->loop_graph = !(lg && lg[0] == '0');
     const char* lv = std::getenv("CAMS_ILU_LEVEL");
     h->ilu_pipelined = !(lv && lv[0] == '1');
-    h->ilu_grid = ilu_pipe_grid(h->g, prop.multiProcessorCount);
-    // One tile per warp for both precisions (with the cross-tile loads
-    // issued ahead of the operand copies it measured faster than 2 x 2 tile
-    // blocks per CTA: 143 against 161 us a 4M-cell FP32 sweep).
-    // CAMS_ILU_CTA=1 forces the tile blocks.
+    h->sms = prop.multiProcessorCount;
+    // blocks of tiles per cluster; CAMS_ILU_CTA=0 runs every tile on its own
     const char* ct = std::getenv("CAMS_ILU_CTA");
-    const bool want = ct && ct[0] == '1';
-    h->ilu_cta = want && ilu_cta_ok(h->g, (int)prop.sharedMemPerBlockOptin);
+    ilu_set_smem();
+    ilu_sweep_smem((int)prop.sharedMemPerBlockOptin);
+    h->ilu_cta = !(ct && ct[0] == '0');
     const char* cc = std::getenv("CAMS_COARSE_CLUSTER");
     h->coarse_cluster = !(cc && cc[0] == '0') &&
                         coarse_cluster_ok(h->c.Nc, (int)prop.sharedMemPerBlockOptin);
@@ -1263,8 +1257,6 @@ int cams_set_schedule(cams_handle* h, int ilu_cta, int coarse_cluster) {
     return fail(h, CAMS_EINVAL, "the level-scheduled sweeps have no tile schedule");
   cudaDeviceProp prop;
   CK(cudaGetDeviceProperties(&prop, h->dev));
-  if (ilu_cta == 1 && !h->ilu_cta && !ilu_cta_ok(h->g, (int)prop.sharedMemPerBlockOptin))
-    return fail(h, CAMS_EINVAL, "2x2 tile blocks do not fit this grid's shared memory");
   if (coarse_cluster == 1 && !h->coarse_cluster &&
       !coarse_cluster_ok(h->c.Nc, (int)prop.sharedMemPerBlockOptin))
     return fail(h, CAMS_EINVAL, "the cluster coarse solve is not available for this coarse grid");

@@ -80,9 +80,9 @@ struct SingleBuffers {
   float *Axu = nullptr, *Ayu = nullptr, *Azu = nullptr;   // transposed couplings (alias Ax.. if symmetric)
   float *Qx = nullptr, *Qy = nullptr, *Qz = nullptr;      // ILU(0) pivot products (nonsymmetric A)
   float* dinv = nullptr;                                  // 1 / ILU(0) pivots
-  float *Lx = nullptr, *Ly = nullptr, *Lz = nullptr;      // scaled couplings, skewed
-  float *Ux = nullptr, *Uy = nullptr, *Uz = nullptr;
-  float *rds = nullptr, *w = nullptr, *z = nullptr;       // smoother vectors, skewed
+  // ILU(0) sweep records (k_sweep.cu): {D^{-1} r, a_{i,i-e_d} / d_i}, {w,
+  // a_{i,i+e_d} / d_i}, and the backward sweep's output
+  float *lo = nullptr, *up = nullptr, *z = nullptr;
   float* d = nullptr;                                     // the correction delta (N)
   float* r = nullptr;                                     // the outer residual rounded to FP32 (N)
   float* P = nullptr;                                     // 8N, slot-major
@@ -132,10 +132,10 @@ struct Buffers {
   double *rc = nullptr, *pc = nullptr;                    // coarse vectors (band order)
   double* ywork = nullptr;                                // forward-solve vector of the global band solve
   double* dinv = nullptr;                                 // 1 / ILU(0) pivots
-  // ILU(0) sweep vectors, skewed tile-major (ilu_skew_len elements each)
-  double *Lx = nullptr, *Ly = nullptr, *Lz = nullptr;     // a_{i,i-e_d} / d_i
-  double *Ux = nullptr, *Uy = nullptr, *Uz = nullptr;     // a_{i,i+e_d} / d_i
-  double *rds = nullptr, *w = nullptr, *z = nullptr;      // D^{-1} r, forward / backward sweeps
+  // ILU(0) sweep records (k_sweep.cu; FP64 handles only; z has ilu_sweep_len
+  // elements, lo and up four times that): {D^{-1} r, a_{i,i-e_d} / d_i}, {w,
+  // a_{i,i+e_d} / d_i}, and the backward sweep's output
+  double *lo = nullptr, *up = nullptr, *z = nullptr;
   int* ctrl = nullptr;                                    // wavefront tickets, abort flag
   double* r = nullptr;                                    // residual (natural order)
   double* cf = nullptr;                                   // correction function Psi (N; FP64 with options.cf)
@@ -242,23 +242,28 @@ cudaError_t launch_prolong_to_p(const Geo& g, const CGeo& c, bool single, Buffer
                                 cudaStream_t s);
 // single: the FP32 smoother of the mixed-precision preconditioner (on
 // A delta = r, vectors in b.f32); otherwise the FP64 smoother on A p = f.
-// sms: the SM count (from ilu_pipe_grid); cta: tiles in 2 x 2 blocks per CTA
-// with shared-memory edges (ilu_cta_ok), else one tile per warp.
+// sms: the SM count; cta: blocks of tiles per thread-block cluster, else one tile
+// per CTA on its own.  launch_ilu_resid resets the tickets of the two sweeps
+// that follow it.  launch_ilu_factor ends with launch_ilu_prepare (the scaled
+// couplings in the sweep layout).
 // nonsym: pivots from the products a_{i,i-e} a_{i-e,i} (b.Qx.., formed here)
-cudaError_t launch_ilu_factor(const Geo& g, Buffers& b, bool pipelined, int sms, bool cta,
-                              bool single, bool nonsym, cudaStream_t s);
+cudaError_t launch_ilu_factor(const Geo& g, Buffers& b, bool pipelined, int sms, bool single,
+                              bool nonsym, cudaStream_t s);
+cudaError_t launch_ilu_prepare(const Geo& g, Buffers& b, bool pipelined, bool single,
+                               cudaStream_t s);
 cudaError_t launch_ilu_resid(const Geo& g, Buffers& b, bool single, cudaStream_t s);
-cudaError_t launch_ilu_sweep(const Geo& g, Buffers& b, bool backward, bool pipelined, int sms,
-                             bool cta, bool single, cudaStream_t s);
+cudaError_t launch_ilu_sweep(const Geo& g, Buffers& b, bool backward, bool pipelined, bool cta,
+                             bool single, cudaStream_t s);
 // x += z after the backward sweep (single: delta in FP32, else p)
 cudaError_t launch_ilu_apply(const Geo& g, Buffers& b, bool single, cudaStream_t s);
-bool ilu_cta_ok(const Geo& g, int max_smem);
+// raise the kernels' shared-memory limits; false when one does not fit
+bool ilu_set_smem();
+bool ilu_sweep_smem(int max_smem);
 cudaError_t launch_add_correction(const Geo& g, Buffers& b, cudaStream_t s);   // p += delta
 int ilu_ctrl_ints(const Geo& g);
-// Rows per wavefront tile (y, z) and the length of a skewed sweep vector.
+// Rows per factorisation tile (y, z), and the length of a sweep vector.
 constexpr int kIluTY = 8, kIluTZ = 4, kIluR = kIluTY * kIluTZ;   // one warp per tile
-long long ilu_skew_len(const Geo& g);
-int ilu_pipe_grid(const Geo& g, int num_sms);
+long long ilu_sweep_len(const Geo& g, bool single);
 cudaError_t launch_wait_selftest(const Geo& g, Buffers& b, cudaStream_t s);
 
 // ---- learned basis surrogate (k_net.cu) ----
