@@ -402,7 +402,7 @@ int cams_net_adam(long long n, float* p, const float* g, float* m, float* v, flo
  * weights and hidden activations are rounded to BF16 (nearest, ties to
  * even); biases, accumulation and the outputs below are FP32.  Device
  * pointers; `work` is caller-owned device memory of at least
- * cams_net_tc_work_bytes(B, S) bytes (cleared and used by the call).  The
+ * cams_net_tc_work_bytes(B, S) bytes (overwritten by the call).  The
  * calls queue their work on `stream` and return when it is done.
  *   conv_forward_tc: one layer, x [B][ci][S^3] -> y [B][co][S^3] FP32
  *                    (ci, co <= CAMS_NET_HID), ReLU when relu != 0.

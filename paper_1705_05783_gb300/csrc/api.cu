@@ -954,7 +954,7 @@ long long tc_work_bytes(int B, int S) {
   return 256 + 2 * ((2 * net_tc_act_elems(B, S, kNetHid) + 255) / 256 * 256);
 }
 
-// Shared driver of the two tensor-core entry points: zero the workspace,
+// Shared driver of the two tensor-core entry points: clear the status word,
 // run `body` on its two activation buffers, wait and read the status word.
 template <class F>
 int run_tc(int B, int S, void* work, long long work_bytes, cudaStream_t s, F body) {
@@ -973,7 +973,7 @@ int run_tc(int B, int S, void* work, long long work_bytes, cudaStream_t s, F bod
   const long long half = (need - 256) / 2;
   void* ta = base + 256;
   void* tb = base + 256 + half;
-  cudaError_t e = cudaMemsetAsync(work, 0, (size_t)need, s);
+  cudaError_t e = cudaMemsetAsync(status, 0, 256, s);   // (the layers write every row that they read)
   if (e == cudaSuccess) e = body(ta, tb, status, prop.multiProcessorCount);
   int st = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, s);

@@ -78,3 +78,28 @@ def test_non_finite_inputs_stay_where_they_are(env):
     # of the last planes have no such pair and stay finite
     assert bool(fin[0, 1].all()) and bool(fin[0, 0, S - 1].all()) and bool(fin[0, 0, :, S - 1].all())
     assert bool(fin[0, 0, :, :, S - 1].all())
+
+
+@pytest.mark.parametrize("S,ci,co", [(5, 12, 32), (6, 32, 32), (5, 32, 8)])
+def test_tensor_core_conv_is_the_same_in_any_batch(env, S, ci, co):
+    """More patches than CTAs (one or two an SM): every CTA runs several, and a
+    patch's result is bit for bit the one it has alone."""
+    torch, cams = env
+    B = 700
+    g = torch.Generator().manual_seed(S)
+    x = torch.randn(B, ci, S, S, S, generator=g).cuda()
+    w = (0.1 * torch.randn(co, ci, 27, generator=g)).cuda()
+    b = torch.randn(co, generator=g).cuda()
+
+    def run(xb):
+        n = xb.shape[0]
+        nb = cams.cams_net_tc_work_bytes(n, S)
+        work = torch.full((nb,), 255, dtype=torch.uint8, device="cuda")   # not cleared by the caller
+        y = torch.full((n, co, S, S, S), float("nan"), device="cuda")
+        assert cams.cams_net_conv_forward_tc(n, S, ci, co, xb, w, b, 1, y, work, nb) == cams.CAMS_OK
+        return y
+
+    y = run(x)
+    assert bool(torch.isfinite(y).all())
+    for k in (0, 1, 151, 152, 303, 304, 456, B - 1):
+        assert torch.equal(run(x[k:k + 1].contiguous())[0], y[k]), k
