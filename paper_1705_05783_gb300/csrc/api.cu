@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "cams_internal.h"
+#include "stencil.h"
 
 using namespace cams;
 
@@ -350,7 +351,10 @@ int alloc_all(cams_handle* h) {
     if (cudaMemset(b.cf, 0, sizeof(double) * (size_t)N) != cudaSuccess)
       return fail(h, CAMS_ECUDA, "cudaMemset failed");
   }
-  AL(b.red, kRedBlocks);
+  AL(b.red, kColBlocks);
+  AL(b.tick, 1);
+  if (cudaMemset(b.tick, 0, sizeof(unsigned)) != cudaSuccess)
+    return fail(h, CAMS_ECUDA, "cudaMemset failed");
   AL(b.scal, 8);
   AL(b.status, 1);
 #undef AL
@@ -362,7 +366,7 @@ void free_all(cams_handle* h) {
   void* ptrs[] = {b.Tx, b.Ty, b.Tz, b.Tbw, b.Tbe, b.p, b.pn, b.rho, b.rhon, b.Ad, b.Ax, b.Ay,
                   b.Az, b.Cacc, b.f, b.eps, b.src, b.Abd, b.Abx, b.Aby, b.Abz, b.snap, b.P,
                   b.ent_of_cell, b.ents, b.flag, b.lscratch, b.loc, b.Acs, b.band, b.perm, b.jxt, b.rc,
-                  b.pc, b.dinv, b.r, b.z, b.red, b.scal, b.status, b.lo, b.up, b.ctrl, b.Lc, b.Lr, b.cblk, b.cdinv, b.cabort, b.fixm,
+                  b.pc, b.dinv, b.r, b.z, b.red, b.tick, b.scal, b.status, b.lo, b.up, b.ctrl, b.Lc, b.Lr, b.cblk, b.cdinv, b.cabort, b.fixm,
                   b.fixc, b.fixv, b.cf, b.Qx, b.Qy, b.Qz, b.Fc, b.ywork, b.lwork,
                   // the transposed couplings are separate arrays only for a nonsymmetric A
                   b.Axu != b.Ax ? b.Axu : nullptr, b.Ayu != b.Ay ? b.Ayu : nullptr,
@@ -708,7 +712,9 @@ int update_operators(cams_handle* h, int force, int* n_rebuilt) {
 }
 
 int residual_norm(cams_handle* h, double* out) {
-  LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, h->b, h->b.p, h->b.r, h->b.red, h->b.scal, h->stream));
+  LoopCtl begin;
+  begin.mode = LoopCtl::kBegin;
+  LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, h->b, h->stream, begin));
   double s2;
   int rc = read_scalar(h, &s2);
   if (rc) return rc;
@@ -759,7 +765,7 @@ int cams_step_direct(cams_handle* h) {
       if (rc) return rc;
     }
     if (s) LAUNCH(CAMS_PROF_UPDATE, launch_add_correction(h->g, b, h->stream));
-    LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, b, b.p, b.r, b.red, b.scal, h->stream));
+    LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, b, h->stream));
   }
   const int fv = h->opt.restriction == 1;
   LAUNCH(CAMS_PROF_RESTRICT, launch_restrict(h->g, h->c, fv, b.r, s, b, h->stream));
@@ -811,28 +817,9 @@ int capture_step(cams_handle* h) {
   return CAMS_OK;
 }
 
-// Device side of the inner loop's stopping test (Sec. 4.1.1): scal[0] holds
-// ||f - A p||^2 of the current iterate (the residual kernel's sum),
-// scal[1] the same at the start of the linearisation, scal[2] the
-// iterations run.  The test is the host loop's, in the same FP64 operations:
-// continue while ||r|| >= lin_rtol ||r^0|| (and finite) and fewer than
-// max_cams iterations have run.
-__global__ void k_loop_begin(double* scal) {
-  scal[1] = scal[0];
-  scal[2] = 0.0;
-}
-__global__ void k_loop_ctrl(cudaGraphConditionalHandle cond, double* scal, int max_cams,
-                            double lin_rtol) {
-  const double its = scal[2] + 1.0;
-  scal[2] = its;
-  const double rn = sqrt(scal[0]), r0 = sqrt(scal[1]);
-  const bool more = its < (double)max_cams && isfinite(rn) && !(rn < lin_rtol * r0);
-  cudaGraphSetConditional(cond, more ? 1u : 0u);
-}
-
 // Capture the inner loop: a graph holding one conditional WHILE node whose
-// body is one C-AMS iteration, the residual norm and k_loop_ctrl (which
-// sets the node's condition).  Like the single-iteration graph it is
+// body is one C-AMS iteration and the residual norm, whose last CTA sets the
+// node's condition.  Like the single-iteration graph it is
 // captured once (every pointer and size is fixed for the handle's life).
 int capture_loop(cams_handle* h) {
   if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
@@ -867,12 +854,12 @@ int capture_loop(cams_handle* h) {
   const long long l0 = lc::mine;
   int rc = cams_step_direct(h);
   if (!rc) {
-    cudaError_t e2 = launch_residual(h->g, h->b, h->b.p, h->b.r, h->b.red, h->b.scal, h->stream);
-    if (e2 == cudaSuccess) {
-      k_loop_ctrl<<<1, 1, 0, h->stream>>>(cond, h->b.scal, h->opt.max_cams, h->opt.lin_rtol);
-      count_launches(1);
-      e2 = cudaGetLastError();
-    }
+    LoopCtl test;
+    test.mode = LoopCtl::kTest;
+    test.max_cams = h->opt.max_cams;
+    test.lin_rtol = h->opt.lin_rtol;
+    test.cond = cond;
+    const cudaError_t e2 = launch_residual(h->g, h->b, h->stream, test);
     if (e2 != cudaSuccess) rc = fail(h, CAMS_ECUDA, std::string("loop graph body: ") + cudaGetErrorString(e2));
   }
   const long long l1 = lc::mine;
@@ -911,9 +898,6 @@ int inner_loop_graph(cams_handle* h, int* its, double* rn) {
       return CAMS_EINVAL;
     }
   }
-  k_loop_begin<<<1, 1, 0, h->stream>>>(h->b.scal);
-  count_launches(1);
-  CK(cudaGetLastError());
   CK(cudaGraphLaunch(h->loop_exec, h->stream));
   double sc[3];
   CK(cudaMemcpyAsync(sc, h->b.scal, sizeof(sc), cudaMemcpyDeviceToHost, h->stream));
@@ -1318,7 +1302,7 @@ int closing_msfv(cams_handle* h) {
     CK(launch_band_fill(h->c, h->mc, 0, b, h->stream));
     CK(launch_band_factor(h->c.Nc, h->mc, 0, b, h->stream));
   }
-  LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, b, b.p, b.r, b.red, b.scal, h->stream));
+  LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, b, h->stream));
   LAUNCH(CAMS_PROF_RESTRICT, launch_restrict(h->g, h->c, 1, b.r, h->single, b, h->stream));
   LAUNCH(CAMS_PROF_COARSE_SOLVE, launch_band_solve(h->c.Nc, h->mc, 0, false, false, b, h->stream));
   LAUNCH(CAMS_PROF_PROLONG, launch_prolong_to_p(h->g, h->c, h->single, b, h->stream));
@@ -1741,7 +1725,7 @@ int cams_get(cams_handle* h, int what, double* dst) {
       break;
     }
     case CAMS_Q_RESIDUAL: {
-      CK(launch_residual(h->g, b, b.p, b.r, b.red, b.scal, s));
+      CK(launch_residual(h->g, b, s));
       CK(cudaMemcpyAsync(dst, b.r, sizeof(double) * N, k, s));
       break;
     }

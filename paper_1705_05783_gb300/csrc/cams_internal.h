@@ -140,6 +140,7 @@ struct Buffers {
   double* r = nullptr;                                    // residual (natural order)
   double* cf = nullptr;                                   // correction function Psi (N; FP64 with options.cf)
   double* red = nullptr;                                  // reduction partials
+  unsigned* tick = nullptr;                               // CTAs that have left theirs
   double* scal = nullptr;                                 // reduced scalars (device)
   int* status = nullptr;                                  // device status word
   SingleBuffers f32;                                      // mixed precision only
@@ -165,10 +166,6 @@ cudaError_t raise_smem_limit(F* func, int bytes) {
 void count_launches(long long n);
 long long launches_total();
 
-// Reductions use a fixed grid so results are bit-reproducible.
-constexpr int kRedBlocks = 1024;
-constexpr int kRedThreads = 256;
-
 // ---- launchers (each returns the launch error) ----
 cudaError_t launch_transmissibility(const Geo& g, double mu, const double* kx, const double* ky,
                                     const double* kz, int dirichlet, Buffers& b, cudaStream_t s);
@@ -183,9 +180,18 @@ cudaError_t launch_add_sources(int n, const int* cell, const double* rate, doubl
                                long long N, cudaStream_t s);
 cudaError_t launch_fix_cells(int n, const int* cell, const double* val, unsigned char* fixm,
                              double* p, long long N, cudaStream_t s);
-cudaError_t launch_sumsq(const double* x, long long N, double* red, double* out, cudaStream_t s);
-cudaError_t launch_residual(const Geo& g, const Buffers& b, const double* p, double* r,
-                            double* red, double* out, cudaStream_t s);
+// The inner loop's part of a residual launch (k_fine.cu): nothing, the start
+// of a linearisation, or the stopping test that sets the loop's condition.
+struct LoopCtl {
+  enum Mode { kNone, kBegin, kTest };
+  int mode = kNone;
+  int max_cams = 0;
+  double lin_rtol = 0.0;
+  cudaGraphConditionalHandle cond{};
+};
+// b.r = f - A b.p (and its FP32 copy in mixed precision), b.scal[0] = ||b.r||^2
+cudaError_t launch_residual(const Geo& g, const Buffers& b, cudaStream_t s,
+                            const LoopCtl& ctl = LoopCtl());
 cudaError_t launch_basis_operator(const Geo& g, const FluidK& fl, int kind, double dt,
                                   const unsigned char* fixm, Buffers& b, cudaStream_t s);
 cudaError_t launch_adapt_flags(const Geo& g, const Entity* ents, int count, double theta,

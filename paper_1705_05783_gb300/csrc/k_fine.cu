@@ -2,11 +2,13 @@
 // linear-system population (a2, Eqs. 3-6 and Eq. 19), the basis operators of
 // Eqs. 8-11, residual SpMV with a fused 2-norm, and deterministic reductions.
 //
-// All kernels are one thread per cell over the x-fastest layout, so every
-// array access of a warp is a coalesced 256-byte run; the six neighbour
-// reads of the 7-point stencil hit L1/L2 (each value is read by up to seven
-// cells).  FP64 throughout.
+// The assembly and the residual march along z (stencil.h); the others are one
+// thread per cell over the x-fastest layout.  Either way every array access
+// of a warp is a coalesced 256-byte run; the neighbour reads of the 7-point
+// stencil hit L1/L2.  FP64 throughout.
 #include "cams_internal.h"
+#include "rcp64.h"
+#include "stencil.h"
 
 namespace cams {
 
@@ -16,40 +18,43 @@ __device__ __forceinline__ void cell_xyz(const Geo& g, long long i, int& x, int&
   xyz_of(g, i, x, y, z);
 }
 
-// Block-wide sum; every thread passes its value, thread 0 gets the total.
-// Fixed shape, fixed order: bit-reproducible for a fixed launch.
-__device__ double block_sum(double v) {
-  __shared__ double sh[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  const int nw = (blockDim.x + 31) >> 5;
-  v = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-  if (wid == 0)
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();
-  return v;
+// 1/d to the last digits; the division itself where the estimate's range
+// ends (subnormal, huge, infinite or not a number).
+__device__ __forceinline__ double rcp_any(double d) {
+  const unsigned ex = ((unsigned)__double2hiint(d) >> 20) & 0x7ffu;
+  if (ex - 1u >= 2043u) return 1.0 / d;
+  return rcp_halley(d);
+}
+
+// TPFA: T = A / (h/(2 lambda_a) + h/(2 lambda_b)), as c k_a (k_b / (k_a +
+// k_b)) with c = 2 A / (h mu): one reciprocal a face instead of five
+// divisions, which were the kernel's time (0.97 ms at 4M cells; an FP64
+// division is a chain of about ten FP64 instructions).  Where that is not
+// finite (both permeabilities zero, or out of range) the formula as it stands
+// decides.
+__device__ __forceinline__ double face_trans(double c, double area, double h, double mu, double ka,
+                                             double kb) {
+  const double t = c * (ka * (kb * rcp_any(ka + kb)));
+  if (isfinite(t)) return t;
+  return area / (h / (2.0 * (ka / mu)) + h / (2.0 * (kb / mu)));
 }
 
 __global__ void k_transmissibility(Geo g, double mu, const double* __restrict__ kx,
                                    const double* __restrict__ ky, const double* __restrict__ kz,
-                                   int dirichlet, double* Tx, double* Ty, double* Tz, double* Tbw,
-                                   double* Tbe) {
+                                   int dirichlet, double cx, double cy, double cz, double* Tx,
+                                   double* Ty, double* Tz, double* Tbw, double* Tbe) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= g.N) return;
   int x, y, z;
   cell_xyz(g, i, x, y, z);
   const double ax = g.dy * g.dz, ay = g.dx * g.dz, az = g.dx * g.dy;
-  const double lx = kx[i] / mu, ly = ky[i] / mu, lz = kz[i] / mu;
-  // TPFA: T = A / (h/(2 lambda_a) + h/(2 lambda_b)) on internal faces
-  Tx[i] = x > 0 ? ax / (g.dx / (2.0 * (kx[i - 1] / mu)) + g.dx / (2.0 * lx)) : 0.0;
-  Ty[i] = y > 0 ? ay / (g.dy / (2.0 * (ky[i - g.sy] / mu)) + g.dy / (2.0 * ly)) : 0.0;
-  Tz[i] = z > 0 ? az / (g.dz / (2.0 * (kz[i - g.sz] / mu)) + g.dz / (2.0 * lz)) : 0.0;
+  Tx[i] = x > 0 ? face_trans(cx, ax, g.dx, mu, kx[i - 1], kx[i]) : 0.0;
+  Ty[i] = y > 0 ? face_trans(cy, ay, g.dy, mu, ky[i - g.sy], ky[i]) : 0.0;
+  Tz[i] = z > 0 ? face_trans(cz, az, g.dz, mu, kz[i - g.sz], kz[i]) : 0.0;
   if (dirichlet) {
     const long long f = y + (long long)g.ny * z;
-    if (x == 0) Tbw[f] = ax / (g.dx / (2.0 * lx));
-    if (x == g.nx - 1) Tbe[f] = ax / (g.dx / (2.0 * lx));
+    if (x == 0) Tbw[f] = cx * kx[i];
+    if (x == g.nx - 1) Tbe[f] = cx * kx[i];
   }
 }
 
@@ -72,116 +77,170 @@ __global__ void k_density(long long N, FluidK fl, const double* __restrict__ p, 
 // leaving i).  A p^{nu+1} = f keeps meaning A dp = -F, so f takes X p^nu over
 // the free columns.  A is then not symmetric: Ax.. hold the row's lower
 // couplings a_{i,i-e}, Axu.. the transposed ones a_{i-e,i}, both at cell i.
-__global__ void k_assemble(Geo g, FluidK fl, double dt, int dirichlet, double pw, double pe,
-                           double rhow, double rhoe, const double* __restrict__ p,
-                           const double* __restrict__ rho, const double* __restrict__ rhon,
-                           const double* __restrict__ Tx, const double* __restrict__ Ty,
-                           const double* __restrict__ Tz, const double* __restrict__ Tbw,
-                           const double* __restrict__ Tbe, const double* __restrict__ src,
-                           const unsigned char* __restrict__ fixm, double* Ad, double* Ax,
-                           double* Ay, double* Az, double* Cacc, double* f, double* eps,
-                           double* red, int full, double* Axu, double* Ayu, double* Azu) {
+//
+// Bound by the FP64 unit, so the instructions are counted: a face takes five
+// (the halves of the face density are applied once, to the sums; powers of
+// two change no digit), the face below along z comes from the cell below, a
+// Dirichlet face takes the place of the missing x face, and the density's
+// reciprocal is the pivots' one (rcp64.h).  400 us at 4M cells (650 with
+// every face formed twice and a division), about 50 instructions a cell.
+struct AsmIn {
+  const double *p, *rho, *rhon, *Tx, *Ty, *Tz, *Tbw, *Tbe, *src;
+  const unsigned char* fixm;
+};
+struct AsmOut {
+  double *Ad, *Ax, *Ay, *Az, *Cacc, *f, *eps, *Axu, *Ayu, *Azu, *red, *scal;
+  unsigned* tick;
+};
+
+template <bool kFix, bool kFull>
+__global__ void __launch_bounds__(kColThreads, 3) k_assemble(
+    Geo g, ColWork w, FluidK fl, double dt, int dirichlet, double pw, double pe, double rhow2,
+    double rhoe2, const __grid_constant__ AsmIn in, const __grid_constant__ AsmOut out) {
+  const double* __restrict__ p = in.p;
+  const double* __restrict__ rho = in.rho;
+  const double phidt = fl.phi * (1.0 / dt), inv_V = 1.0 / g.V, half_inv_V = 0.5 * inv_V;
+  const double vphidt = g.V * phidt;
+  // d rho / dp: c rho for the exponential law, rho0 c for the linear one
+  const double dlin = fl.rho0 * fl.c;
+  const double ccst = vphidt * (fl.law == 0 ? fl.c : dlin);
   double e2 = 0.0;
-  const double inv_dt = 1.0 / dt, inv_V = 1.0 / g.V;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N;
-       i += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    cell_xyz(g, i, x, y, z);
-    const double pi = p[i], ri = rho[i];
-    const bool fi = fixm && fixm[i];
-    double flux = 0.0, dsum = 0.0, rhsb = 0.0;
-    // Reading R4: face density = arithmetic mean of the two cell densities
-#define CAMS_FACE(cond, T, j, lowslot)                              \
-    if (cond) {                                                     \
-      const double w = (T) * (0.5 * (ri + rho[j]));                 \
-      dsum += w;                                                    \
-      flux += w * (pi - p[j]);                                      \
-      if (fixm && (fi || fixm[j])) {                                \
-        if (!fi) rhsb += w * p[j];                                  \
-      } else {                                                      \
-        lowslot;                                                    \
-      }                                                             \
+  for (unsigned w0 = blockIdx.x; w0 < w.pieces; w0 += gridDim.x) {
+    const unsigned seg = w0 / w.tiles;
+    const long long j = (long long)(w0 - seg * w.tiles) * kColThreads + threadIdx.x;
+    if (j >= g.sz) continue;
+    const unsigned y = (unsigned)j / (unsigned)g.nx, x = (unsigned)j - y * (unsigned)g.nx;
+    const bool xl = x > 0, xu = x + 1 < (unsigned)g.nx, yl = y > 0, yu = y + 1 < (unsigned)g.ny;
+    const int z0 = (int)seg * w.planes, z1 = min(z0 + w.planes, g.nz);
+    long long i = j + g.sz * z0;
+    double pi = p[i], ri = rho[i];
+    bool fi = kFix && in.fixm[i];
+    // the face below: twice its coefficient, p_below - p_i, and the cell's data
+    double wz = 0.0, dz = 0.0, pz = 0.0, rz = 0.0, Tzl = 0.0;
+    bool fz = false;
+    if (z0 > 0) {
+      rz = rho[i - g.sz];
+      Tzl = in.Tz[i];
+      wz = Tzl * (ri + rz);
+      pz = p[i - g.sz];
+      dz = pz - pi;
+      fz = kFix && in.fixm[i - g.sz];
     }
-    double ax = 0.0, ay = 0.0, az = 0.0;
-    CAMS_FACE(x > 0, Tx[i], i - 1, ax = -w)
-    CAMS_FACE(x < g.nx - 1, Tx[i + 1], i + 1, (void)0)
-    CAMS_FACE(y > 0, Ty[i], i - g.sy, ay = -w)
-    CAMS_FACE(y < g.ny - 1, Ty[i + g.sy], i + g.sy, (void)0)
-    CAMS_FACE(z > 0, Tz[i], i - g.sz, az = -w)
-    CAMS_FACE(z < g.nz - 1, Tz[i + g.sz], i + g.sz, (void)0)
-#undef CAMS_FACE
-    if (dirichlet) {
-      const long long fi2 = y + (long long)g.ny * z;
-      if (x == 0) {
-        const double wb = Tbw[fi2] * rhow;
-        dsum += wb; flux += wb * (pi - pw); rhsb += wb * pw;
+    for (int z = z0; z < z1; ++z, i += g.sz) {
+      const bool zu = z + 1 < g.nz;
+      const long long fb = y + (long long)g.ny * z;
+      // every load of the cell, before the first use
+      const double rn = in.rhon[i];
+      double Txl, Txu, pxl, pxu, rxl, rxu;
+      if (xl) { Txl = in.Tx[i]; pxl = p[i - 1]; rxl = rho[i - 1]; }
+      else { Txl = dirichlet ? in.Tbw[fb] : 0.0; pxl = dirichlet ? pw : 0.0; rxl = 0.0; }
+      if (xu) { Txu = in.Tx[i + 1]; pxu = p[i + 1]; rxu = rho[i + 1]; }
+      else { Txu = dirichlet ? in.Tbe[fb] : 0.0; pxu = dirichlet ? pe : 0.0; rxu = 0.0; }
+      const double Tyl = yl ? in.Ty[i] : 0.0, pyl = yl ? p[i - g.sy] : 0.0;
+      const double ryl = yl ? rho[i - g.sy] : 0.0;
+      const double Tyu = yu ? in.Ty[i + g.sy] : 0.0, pyu = yu ? p[i + g.sy] : 0.0;
+      const double ryu = yu ? rho[i + g.sy] : 0.0;
+      const double Tzu = zu ? in.Tz[i + g.sz] : 0.0, pzu = zu ? p[i + g.sz] : 0.0;
+      const double rzu = zu ? rho[i + g.sz] : 0.0;
+      const double q = in.src ? in.src[i] * inv_V : 0.0;
+      bool fxl = false, fxu = false, fyl = false, fyu = false, fzu = false;
+      if constexpr (kFix) {
+        fxl = xl && in.fixm[i - 1]; fxu = xu && in.fixm[i + 1];
+        fyl = yl && in.fixm[i - g.sy]; fyu = yu && in.fixm[i + g.sy];
+        fzu = zu && in.fixm[i + g.sz];
       }
-      if (x == g.nx - 1) {
-        const double wb = Tbe[fi2] * rhoe;
-        dsum += wb; flux += wb * (pi - pe); rhsb += wb * pe;
+      // Reading R4: face density = arithmetic mean of the two cell densities
+      // (w.. hold twice the face's coefficient; the prescribed density of a
+      // Dirichlet face is given doubled)
+      const double sxl = ri + rxl, sxu = ri + rxu;
+      const double wxl = Txl * (xl ? sxl : rhow2), wxu = Txu * (xu ? sxu : rhoe2);
+      const double wyl = Tyl * (ri + ryl), wyu = Tyu * (ri + ryu), wzu = Tzu * (ri + rzu);
+      // absent faces: their difference counts as zero whatever p_i is
+      const bool bx = dirichlet != 0;
+      const double dxl = xl || bx ? pi - pxl : 0.0, dxu = xu || bx ? pi - pxu : 0.0;
+      const double dyl = yl ? pi - pyl : 0.0, dyu = yu ? pi - pyu : 0.0;
+      const double dzu = zu ? pi - pzu : 0.0;
+      double d2 = wxl + wxu;
+      d2 += wyl; d2 += wyu; d2 += wz; d2 += wzu;
+      double fl2 = wxl * dxl;
+      fl2 += wxu * dxu; fl2 += wyl * dyl; fl2 += wyu * dyu; fl2 -= wz * dz; fl2 += wzu * dzu;
+      double rhs2 = 0.0;
+      if (bx && !(kFix && fi)) {
+        if (!xl) rhs2 += wxl * pw;
+        if (!xu) rhs2 += wxu * pe;
       }
-    }
-    const double rn = rhon[i];
-    // d rho / dp: c rho for the exponential law (rho_i already holds
-    // rho0 exp(c p_i)), rho0 eta for the linear one
-    const double drho = fl.law == 0 ? fl.c * ri : fl.rho0 * fl.c;
-    // FP64 divisions are long dependent sequences on this GPU: one per cell
-    const double rinv = 1.0 / ri;
-    const double phidt = fl.phi * inv_dt;
-    // Eq. 4 with d phi/dp = 0, then the row scaling V rho (Reading R7)
-    const double cc = phidt * rn * drho * rinv * rinv;
-    const double C = g.V * ri * cc;
-    const double q = src ? src[i] * inv_V : 0.0;
-    const double b = -phidt + phidt * rn * rinv + q;   // Eq. 5
-    double xdiag = 0.0, xp = 0.0;
-    if (full) {
-      double axu = 0.0, ayu = 0.0, azu = 0.0;
-#define CAMS_JFACE(cond, T, j, lowslot)                                        \
-      if (cond) {                                                              \
-        const double h = 0.5 * (T) * (pi - p[j]);                              \
-        xdiag += h * drho;                                                     \
-        if (!(fixm && (fi || fixm[j]))) {                                      \
-          const double drj = fl.law == 0 ? fl.c * rho[j] : fl.rho0 * fl.c;     \
-          xp += h * drj * p[j];                                                \
-          lowslot;                                                             \
-        }                                                                      \
+      const bool cut = kFix && fi;
+      if constexpr (kFix) {
+        if (!fi) {
+          if (fxl) rhs2 += wxl * pxl;
+          if (fxu) rhs2 += wxu * pxu;
+          if (fyl) rhs2 += wyl * pyl;
+          if (fyu) rhs2 += wyu * pyu;
+          if (fz) rhs2 += wz * pz;
+          if (fzu) rhs2 += wzu * pzu;
+        }
       }
-      // a lower face also gives the transposed entry a_{j,i} = -w - h rho'_i
-      CAMS_JFACE(x > 0, Tx[i], i - 1,
-                 (ax += h * drj, axu = -(Tx[i] * (0.5 * (ri + rho[i - 1]))) - h * drho))
-      CAMS_JFACE(x < g.nx - 1, Tx[i + 1], i + 1, (void)0)
-      CAMS_JFACE(y > 0, Ty[i], i - g.sy,
-                 (ay += h * drj, ayu = -(Ty[i] * (0.5 * (ri + rho[i - g.sy]))) - h * drho))
-      CAMS_JFACE(y < g.ny - 1, Ty[i + g.sy], i + g.sy, (void)0)
-      CAMS_JFACE(z > 0, Tz[i], i - g.sz,
-                 (az += h * drj, azu = -(Tz[i] * (0.5 * (ri + rho[i - g.sz]))) - h * drho))
-      CAMS_JFACE(z < g.nz - 1, Tz[i + g.sz], i + g.sz, (void)0)
+      // FP64 divisions are long dependent sequences on this GPU
+      const double rinv = rcp_any(ri);
+      // Eq. 4 with d phi/dp = 0, then the row scaling V rho (Reading R7):
+      // C = V rho phi/dt rho^n rho' / rho^2
+      const double t = rn * rinv;
+      const double C = ccst * (fl.law == 0 ? rn : t);
+      const double b = fma(phidt, t, q - phidt);         // Eq. 5
+      const double flux = fl2 * half_inv_V;              // over V
+      double xdiag = 0.0, xp = 0.0;
+      double ax = xl && !cut && !fxl ? -0.5 * wxl : 0.0;
+      double ay = yl && !cut && !fyl ? -0.5 * wyl : 0.0;
+      double az = !cut && !fz && z > 0 ? -0.5 * wz : 0.0;
+      if constexpr (kFull) {
+        const double drho = fl.law == 0 ? fl.c * ri : dlin;
+        double axu = 0.0, ayu = 0.0, azu = 0.0;
+#define CAMS_JFACE(cond, T, dp, fj, pj, rj, lowslot)                           \
+        if (cond) {                                                            \
+          const double h = 0.5 * (T) * (dp);                                   \
+          xdiag += h * drho;                                                   \
+          if (!(kFix && (fi || (fj)))) {                                       \
+            const double drj = fl.law == 0 ? fl.c * (rj) : dlin;               \
+            xp += h * drj * (pj);                                              \
+            lowslot;                                                           \
+          }                                                                    \
+        }
+        // a lower face also gives the transposed entry a_{j,i} = -w - h rho'_i
+        CAMS_JFACE(xl, Txl, dxl, fxl, pxl, rxl, (axu = ax - h * drho, ax += h * drj))
+        CAMS_JFACE(xu, Txu, dxu, fxu, pxu, rxu, (void)0)
+        CAMS_JFACE(yl, Tyl, dyl, fyl, pyl, ryl, (ayu = ay - h * drho, ay += h * drj))
+        CAMS_JFACE(yu, Tyu, dyu, fyu, pyu, ryu, (void)0)
+        CAMS_JFACE(z > 0, Tzl, -dz, fz, pz, rz, (azu = az - h * drho, az += h * drj))
+        CAMS_JFACE(zu, Tzu, dzu, fzu, pzu, rzu, (void)0)
 #undef CAMS_JFACE
-      xdiag -= flux * drho * rinv;
-      Axu[i] = axu; Ayu[i] = ayu; Azu[i] = azu;
-    }
-    Ax[i] = ax; Ay[i] = ay; Az[i] = az;
-    Cacc[i] = C;
-    double e = 0.0;
-    if (fi) {
-      Ad[i] = 1.0;
-      f[i] = pi;
-    } else {
-      double fv = g.V * ri * b + rhsb + C * pi;
-      if (full) {
-        Ad[i] = C + dsum + xdiag;
-        fv += xdiag * pi + xp;
-      } else {
-        Ad[i] = C + dsum;
+        xdiag -= 0.5 * fl2 * drho * rinv;
+        out.Axu[i] = axu; out.Ayu[i] = ayu; out.Azu[i] = azu;
       }
-      f[i] = fv;
-      e = q - phidt + phidt * rn * rinv - flux * inv_V * rinv;  // Eq. 19
+      out.Ax[i] = ax; out.Ay[i] = ay; out.Az[i] = az;
+      out.Cacc[i] = C;
+      double e = 0.0;
+      if (cut) {
+        out.Ad[i] = 1.0;
+        out.f[i] = pi;
+      } else {
+        double fv = fma(g.V * ri, b, C * pi);
+        if (kFix || bx) fv += 0.5 * rhs2;
+        double ad = fma(0.5, d2, C);
+        if constexpr (kFull) {
+          ad += xdiag;
+          fv += xdiag * pi + xp;
+        }
+        out.Ad[i] = ad;
+        out.f[i] = fv;
+        e = fma(-flux, rinv, b);                         // Eq. 19
+      }
+      out.eps[i] = e;
+      e2 += e * e;
+      wz = wzu; dz = dzu; pz = pi; fz = fi; rz = ri; Tzl = Tzu;
+      pi = pzu; ri = rzu; fi = fzu;
     }
-    eps[i] = e;
-    e2 += e * e;
   }
-  const double s = block_sum(e2);
-  if (threadIdx.x == 0) red[blockIdx.x] = s;
+  finish_sum(block_sum(e2), out.red, out.tick, out.scal);
 }
 
 // Prescribed cells in list order (a repeated cell keeps its last value):
@@ -208,56 +267,34 @@ __global__ void k_add_sources(int n, const int* __restrict__ cell, const double*
   }
 }
 
-__global__ void k_sumsq_partial(const double* __restrict__ x, long long N, double* red) {
-  double s = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x)
-    s += x[i] * x[i];
-  s = block_sum(s);
-  if (threadIdx.x == 0) red[blockIdx.x] = s;
-}
-
-__global__ void k_finish_sum(const double* __restrict__ red, int n, double* out) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += red[i];
-  s = block_sum(s);
-  if (threadIdx.x == 0) out[0] = s;
-}
-
-// r = f - A p and per-block sums of r^2 (kNS: Axu.. hold the couplings to
-// the upper neighbours; otherwise A is symmetric and Ax.. serve both).  Warps take whole
-// x-rows (lanes along x, coalesced), so the cell coordinates cost one
-// division per row.  r32 (null unless wanted): r rounded to FP32 once, for
-// the mixed preconditioner's restriction and smoothing steps, which would
+// r = f - A p and ||r||^2, with the inner loop's bookkeeping by the thread
+// that completes the sum.  r32 (null unless wanted): r rounded to FP32 once,
+// for the mixed preconditioner's restriction and smoothing steps, which would
 // otherwise each round it again (an FP64-unit conversion per cell).
-template <bool kNS>
-__global__ void k_residual(Geo g, const double* __restrict__ Ad, const double* __restrict__ Ax,
-                           const double* __restrict__ Ay, const double* __restrict__ Az,
-                           const double* __restrict__ Axu, const double* __restrict__ Ayu,
-                           const double* __restrict__ Azu, const double* __restrict__ f,
-                           const double* __restrict__ p, double* r, float* r32, double* red) {
-  double s2 = 0.0;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const unsigned rows = (unsigned)g.ny * (unsigned)g.nz;
-  for (unsigned row = blockIdx.x * nw + warp; row < rows; row += gridDim.x * nw) {
-    const int y = (int)(row % (unsigned)g.ny), z = (int)(row / (unsigned)g.ny);
-    const long long base = g.sy * y + g.sz * z;
-    for (int x = lane; x < g.nx; x += 32) {
-      const long long i = base + x;
-      double a = f[i] - Ad[i] * p[i];
-      if (x > 0) a -= Ax[i] * p[i - 1];
-      if (x < g.nx - 1) a -= (kNS ? Axu : Ax)[i + 1] * p[i + 1];
-      if (y > 0) a -= Ay[i] * p[i - g.sy];
-      if (y < g.ny - 1) a -= (kNS ? Ayu : Ay)[i + g.sy] * p[i + g.sy];
-      if (z > 0) a -= Az[i] * p[i - g.sz];
-      if (z < g.nz - 1) a -= (kNS ? Azu : Az)[i + g.sz] * p[i + g.sz];
-      if (r) r[i] = a;
-      if (r32) r32[i] = (float)a;
-      s2 += a * a;
-    }
+//
+// The loop's stopping test (Sec. 4.1.1): scal[0] is ||f - A p||^2 of the
+// current iterate, scal[1] the same at the start of the linearisation,
+// scal[2] the iterations run.  The test is the host loop's, in the same FP64
+// operations: continue while ||r|| >= lin_rtol ||r^0|| (and finite) and fewer
+// than max_cams iterations have run.
+__global__ void __launch_bounds__(kColThreads, 4) k_residual(
+    Geo g, ColWork w, const double* __restrict__ Ad, const double* __restrict__ Ax,
+    const double* __restrict__ Ay, const double* __restrict__ Az, const double* __restrict__ Axu,
+    const double* __restrict__ Ayu, const double* __restrict__ Azu, const double* __restrict__ f,
+    const double* __restrict__ p, double* r, float* r32, double* red, unsigned* tick, double* scal,
+    LoopCtl ctl) {
+  const double s2 = block_sum(residual_columns(g, w, Ad, Ax, Ay, Az, Axu, Ayu, Azu, f, p, r, r32));
+  if (!finish_sum(s2, red, tick, scal)) return;
+  if (ctl.mode == LoopCtl::kBegin) {
+    scal[1] = scal[0];
+    scal[2] = 0.0;
+  } else if (ctl.mode == LoopCtl::kTest) {
+    const double its = scal[2] + 1.0;
+    scal[2] = its;
+    const double rn = sqrt(scal[0]), r0 = sqrt(scal[1]);
+    const bool more = its < (double)ctl.max_cams && isfinite(rn) && !(rn < ctl.lin_rtol * r0);
+    cudaGraphSetConditional(ctl.cond, more ? 1u : 0u);
   }
-  s2 = block_sum(s2);
-  if (threadIdx.x == 0) red[blockIdx.x] = s2;
 }
 
 // Basis operators A_b (Eqs. 8-11, Reading R10: internal faces only).
@@ -311,8 +348,11 @@ inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
 cudaError_t launch_transmissibility(const Geo& g, double mu, const double* kx, const double* ky,
                                     const double* kz, int dirichlet, Buffers& b, cudaStream_t s) {
-  k_transmissibility<<<blocks_for(g.N, 256), 256, 0, s>>>(g, mu, kx, ky, kz, dirichlet, b.Tx,
-                                                          b.Ty, b.Tz, b.Tbw, b.Tbe); count_launches(1);
+  k_transmissibility<<<blocks_for(g.N, 256), 256, 0, s>>>(
+      g, mu, kx, ky, kz, dirichlet, 2.0 * (g.dy * g.dz) / (g.dx * mu),
+      2.0 * (g.dx * g.dz) / (g.dy * mu), 2.0 * (g.dx * g.dy) / (g.dz * mu), b.Tx, b.Ty, b.Tz,
+      b.Tbw, b.Tbe);
+  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -325,15 +365,18 @@ cudaError_t launch_density(const Geo& g, const FluidK& fl, const double* p, doub
 cudaError_t launch_assemble(const Geo& g, const FluidK& fl, double dt, int dirichlet, double pw,
                             double pe, const unsigned char* fixm, bool full, Buffers& b,
                             cudaStream_t s) {
-  FluidK f2 = fl;
   const double rhow = fl.law == 0 ? fl.rho0 * std::exp(fl.c * pw) : fl.rho0 * (1.0 + fl.c * pw);
   const double rhoe = fl.law == 0 ? fl.rho0 * std::exp(fl.c * pe) : fl.rho0 * (1.0 + fl.c * pe);
-  k_assemble<<<kRedBlocks, kRedThreads, 0, s>>>(g, f2, dt, dirichlet, pw, pe, rhow, rhoe, b.p,
-                                                b.rho, b.rhon, b.Tx, b.Ty, b.Tz, b.Tbw, b.Tbe,
-                                                b.src, fixm, b.Ad, b.Ax, b.Ay, b.Az, b.Cacc, b.f,
-                                                b.eps, b.red, full ? 1 : 0, b.Axu, b.Ayu,
-                                                b.Azu); count_launches(1);
-  k_finish_sum<<<1, 1024, 0, s>>>(b.red, kRedBlocks, b.scal); count_launches(1);
+  const AsmIn in{b.p, b.rho, b.rhon, b.Tx, b.Ty, b.Tz, b.Tbw, b.Tbe, b.src, fixm};
+  const AsmOut out{b.Ad, b.Ax, b.Ay, b.Az, b.Cacc, b.f, b.eps, b.Axu, b.Ayu, b.Azu, b.red, b.scal,
+                   b.tick};
+  auto* kern = fixm ? (full ? k_assemble<true, true> : k_assemble<true, false>)
+                    : (full ? k_assemble<false, true> : k_assemble<false, false>);
+  const ColWork w = col_work(g);
+  kern<<<col_grid(w), kColThreads, 0, s>>>(g, w, fl, dt, dirichlet, pw, pe,
+                                           dirichlet ? 2.0 * rhow : 0.0,
+                                           dirichlet ? 2.0 * rhoe : 0.0, in, out);
+  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -349,24 +392,12 @@ cudaError_t launch_fix_cells(int n, const int* cell, const double* val, unsigned
   return cudaGetLastError();
 }
 
-cudaError_t launch_sumsq(const double* x, long long N, double* red, double* out, cudaStream_t s) {
-  k_sumsq_partial<<<kRedBlocks, kRedThreads, 0, s>>>(x, N, red); count_launches(1);
-  k_finish_sum<<<1, 1024, 0, s>>>(red, kRedBlocks, out); count_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_residual(const Geo& g, const Buffers& b, const double* p, double* r,
-                            double* red, double* out, cudaStream_t s) {
-  // the FP32 copy goes with the handle's own residual vector (mixed precision)
-  float* r32 = (r && r == b.r) ? b.f32.r : nullptr;
-  if (b.Axu != b.Ax)
-    k_residual<true><<<kRedBlocks, kRedThreads, 0, s>>>(g, b.Ad, b.Ax, b.Ay, b.Az, b.Axu, b.Ayu,
-                                                        b.Azu, b.f, p, r, r32, red);
-  else
-    k_residual<false><<<kRedBlocks, kRedThreads, 0, s>>>(g, b.Ad, b.Ax, b.Ay, b.Az, b.Axu, b.Ayu,
-                                                         b.Azu, b.f, p, r, r32, red);
+cudaError_t launch_residual(const Geo& g, const Buffers& b, cudaStream_t s, const LoopCtl& ctl) {
+  const ColWork w = col_work(g);
+  k_residual<<<col_grid(w), kColThreads, 0, s>>>(g, w, b.Ad, b.Ax, b.Ay, b.Az, b.Axu, b.Ayu, b.Azu,
+                                                 b.f, b.p, b.r, b.f32.r, b.red, b.tick, b.scal,
+                                                 ctl);
   count_launches(1);
-  k_finish_sum<<<1, 1024, 0, s>>>(red, kRedBlocks, out); count_launches(1);
   return cudaGetLastError();
 }
 

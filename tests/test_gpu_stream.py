@@ -1,0 +1,90 @@
+"""The streaming FP64 kernels at the edges of their split of the grid: pieces
+of 256 (or 1024) columns, runs of planes that share a face, one cluster for
+the smallest calls.
+
+Tolerances: a residual is a sum of eight products in another order, a few
+ulps of the terms' magnitudes; a matrix entry is a product of sums of two,
+1e-13 relative to the largest entry as in the small-grid parity tests."""
+import numpy as np
+import pytest
+
+import oracle
+
+from _cases import gpu_handle, make_case, matrix_from_gpu
+from test_gpu_parity import _rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cams():
+    from paper_1705_05783_gb300 import cams
+    return cams
+
+
+# one cell; one piece; the last cluster size and the first grid beyond it;
+# one column; flat, thin and ragged grids; two and more planes a run
+@pytest.mark.parametrize("n", [(1, 1, 1), (40, 40, 1), (32, 32, 32), (32, 32, 33), (1025, 1, 3), (1, 1, 77),
+                               (3, 257, 5), (181, 181, 1), (97, 101, 103), (128, 65, 130)])
+def test_noalloc_residual_over_the_split(cams, n):
+    import torch
+    nx, ny, nz = n
+    N = nx * ny * nz
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    d, ax, ay, az, f, p = (torch.rand(nz, ny, nx, generator=gen, device="cuda", dtype=torch.float64) - 0.3
+                           for _ in range(6))
+    want, mag = f - d * p, f.abs() + (d * p).abs()
+    for a, dim in ((ax, 2), (ay, 1), (az, 0)):
+        m = a.shape[dim]
+        c = a.narrow(dim, 1, m - 1) if m > 1 else a.narrow(dim, 0, 0)
+        lo, up = p.narrow(dim, 0, max(m - 1, 0)), p.narrow(dim, 1, m - 1) if m > 1 else p.narrow(dim, 0, 0)
+        want.narrow(dim, 1 if m > 1 else 0, m - 1).sub_(c * lo)
+        mag.narrow(dim, 1 if m > 1 else 0, m - 1).add_((c * lo).abs())
+        want.narrow(dim, 0, m - 1).sub_(c * up)
+        mag.narrow(dim, 0, m - 1).add_((c * up).abs())
+        a.narrow(dim, 0, 1).fill_(float("nan"))          # outside the grid: never used
+    r = torch.full((N,), float("nan"), device="cuda", dtype=torch.float64)
+    args = [v.reshape(-1).contiguous() for v in (d, ax, ay, az, f, p)]
+    code, norm = cams.cams_residual_norm_noalloc(nx, ny, nz, *args, r, torch.cuda.current_stream().cuda_stream)
+    assert code == cams.CAMS_OK
+    assert bool(((r - want.reshape(-1)).abs() <= 32 * np.finfo(float).eps * mag.reshape(-1)).all())
+    assert abs(norm - r.norm().item()) <= 1e-12 * norm
+    again = cams.cams_residual_norm_noalloc(nx, ny, nz, *args, None, torch.cuda.current_stream().cuda_stream)
+    assert again == (cams.CAMS_OK, norm)
+
+
+@pytest.mark.parametrize("jacobian", [0, 1])
+@pytest.mark.parametrize("case", [dict(name="3d-200x200x100", nx=140, ny=120, nz=65, coarse=(10, 10, 5)),
+                                  dict(name="3d-100x100x50-wells", nx=140, ny=120, nz=65, coarse=(10, 10, 5)),
+                                  dict(name="3d-64x64x64-lines-a5", nx=112, ny=104, nz=88)],
+                         ids=["dirichlet", "wells", "lines"])
+def test_assembly_on_runs_of_planes(cams, case, jacobian):
+    case = make_case(**case)
+    h, bc, keep = gpu_handle(case, jacobian=jacobian)
+    try:
+        N, nx, ny = case.N, case.w.nx, case.w.ny
+        rng = np.random.default_rng(3)
+        p_nu, p_n = rng.uniform(-0.2, 1.1, N), rng.uniform(-0.2, 1.1, N)
+        if len(case.inp["fix_cell"]):
+            p_nu[case.inp["fix_cell"]] = case.inp["fix_value"]
+        eps = cams.cams_assemble(h, p_nu, p_n, case.inp["dt"], bc)
+        lin = oracle.assemble(case.pb, p_nu, p_n, case.inp["dt"], **(dict(full_jacobian=True) if jacobian else {}))
+        A = lin.A.tocsr()
+        i = np.arange(N)
+        got = matrix_from_gpu(h, N)
+        assert _rel(got[0], A.diagonal()) < 1e-13
+        up = cams.cams_get(h, cams.CAMS_Q_MATRIX_UPPER, np.zeros(3 * N)) if jacobian else None
+        for k, (off, ok) in enumerate(((1, i % nx > 0), (nx, (i // nx) % ny > 0), (nx * ny, i // (nx * ny) > 0))):
+            lo = np.zeros(N)
+            lo[off:] = A.diagonal(-off)
+            assert not lo[~ok].any()
+            assert _rel(got[1 + k], lo) < 1e-13
+            if jacobian:
+                tr = np.zeros(N)
+                tr[off:] = A.diagonal(off)
+                assert _rel(up[k * N:(k + 1) * N], tr) < 1e-13
+        assert _rel(cams.cams_get(h, cams.CAMS_Q_RHS, np.zeros(N)), lin.f) < 1e-12
+        want = np.linalg.norm(lin.eps)
+        assert abs(eps - want) <= 1e-11 * want
+    finally:
+        cams.cams_destroy(h)
