@@ -44,43 +44,61 @@ __device__ __forceinline__ void dual_range(const CGeo& c, const Geo& g, int d, i
   hi = j == c.nc[d] ? n - 1 : j * c.b[d] + c.o[d] - 1;
 }
 
-// Warp sums in the accumulation type TA, the sum over warps in FP64.
+// Sums of K values (a power of two) over the lanes of a warp; lane l returns
+// sum l / (32 / K).  Each step halves the values a lane keeps and hands the
+// others to its partner, K - 1 + log2(32 / K) additions in place of 5 K: an
+// FP64 addition holds the sub-partition's unit for about 64 cycles, and with
+// 8 sums a block these were half of the restriction's time.  The pairs are
+// those of a tree over the lanes, so the sums are the same digits.
 template <int K, class TA>
-__device__ void block_sum_k(TA (&v)[K], double* sh /* K*32 */, double* out) {
+__device__ __forceinline__ TA warp_fold(TA* v) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int n = K / 2; n >= 1; n >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const TA send = up ? v[k] : v[k + n];
+      const TA keep = up ? v[k + n] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    o >>= 1;
+  }
+  for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
+// Warp sums in the accumulation type TA, the sum over warps in FP64, in
+// warp order.
+template <int K, class TA>
+__device__ void block_sum_k(TA (&v)[K], double* sh /* K*8: at most 8 warps */, double* out) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if constexpr (sizeof(TA) == 4) {
-    // FP32 sums: lane k % 32 collects sum k, so that each warp converts its
-    // sums to FP64 in ceil(K / 32) instructions instead of K (a conversion is
-    // an FP64-unit instruction, as slow with one active lane as with 32)
-    constexpr int kW = (K + 31) / 32;
-    TA mine[kW];
-#pragma unroll
-    for (int w = 0; w < kW; ++w) mine[w] = TA(0);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      TA t = v[k];
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      t = __shfl_sync(0xffffffffu, t, 0);
-      if (lane == k % 32) mine[k / 32] = t;
-    }
-#pragma unroll
-    for (int w = 0; w < kW; ++w)
-      if (32 * w + lane < K) sh[(32 * w + lane) * 32 + wid] = (double)mine[w];
-  } else {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      TA t = v[k];
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      if (lane == 0) sh[k * 32 + wid] = (double)t;
-    }
+  constexpr int kLo = K >= 32 ? 32 : K, kHi = K - kLo;
+  static_assert((kLo & (kLo - 1)) == 0 && (kHi & (kHi - 1)) == 0, "powers of two");
+  {
+    const TA t = warp_fold<kLo>(v);
+    if (lane % (32 / kLo) == 0) sh[(lane / (32 / kLo)) * 8 + wid] = (double)t;
+  }
+  if constexpr (kHi > 0) {
+    const TA t = warp_fold<kHi>(v + kLo);
+    if (lane % (32 / kHi) == 0) sh[(kLo + lane / (32 / kHi)) * 8 + wid] = (double)t;
   }
   __syncthreads();
   for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += sh[k * 32 + w];
+    double t = sh[k * 8];
+    for (int w = 1; w < nw; ++w) t += sh[k * 8 + w];
     out[k] = t;
   }
   __syncthreads();
+}
+
+// Threads of the kernels that take one dual (or primal) block a CTA: one per
+// cell up to 256.  The sums of a warp without cells would cost as much as
+// those of a full one.
+inline int block_threads(const CGeo& c) {
+  const long long cells = (long long)c.b[0] * c.b[1] * c.b[2];
+  return cells >= 256 ? 256 : (int)((cells + 31) / 32 * 32);
 }
 
 __device__ __forceinline__ int sym_idx(int s, int t) {   // upper triangle of 8x8, s <= t
@@ -117,7 +135,7 @@ __global__ void __launch_bounds__(256) k_galerkin_fe_local(
     Geo g, CGeo c, const TP* __restrict__ P, const double* __restrict__ Ad,
     const double* __restrict__ Ax, const double* __restrict__ Ay, const double* __restrict__ Az,
     double* loc) {
-  __shared__ double sh[36 * 32];
+  __shared__ double sh[36 * 8];
   const int ndx = c.nc[0] + 1, ndy = c.nc[1] + 1;
   const int D = blockIdx.x;
   const int j[3] = {D % ndx, (D / ndx) % ndy, D / (ndx * ndy)};
@@ -904,7 +922,11 @@ __global__ void __launch_bounds__(256) k_ldlt_solve(int N, int m, const double* 
 // factorisation.  k_coarse_solve_cluster deals the blocks round-robin to the
 // kCC CTAs of one cluster; each CTA keeps a copy of y and x in shared memory
 // (kNotReady until written) and the owner of a block stores its values into
-// every CTA's copy through distributed shared memory.
+// every CTA's copy through distributed shared memory.  The chain from block to
+// block bounds it (1000 unknowns, half-width 111, FP64: 69 us), so whatever
+// does not depend on another block's values is in registers before they
+// arrive: with the factor's entries loaded after each wait, two trips to L2 a
+// block, it took 100.
 constexpr int kCB = 32;                      // rows per block
 constexpr int kCBlocks = 3;                  // per block: L_JJ^{-1}, M_J, M'_J
 constexpr int kCC = 8;                       // CTAs per cluster
@@ -917,59 +939,58 @@ __device__ __forceinline__ double lower_at(const double* Lc, int N, int m, int r
   return (r < N && c >= 0 && r > c && r - c <= m) ? Lc[(long long)c * (m + 1) + (r - c)] : 0.0;
 }
 
-// One CTA per block J: blk[J] = { L_JJ^{-1}, M_J, M'_J } (kCB x kCB each,
-// row-major), dinv[i] = 1 / d_i.  Rows past N act as identity rows.
+// Three CTAs per block J, one for each of blk[J] = { L_JJ^{-1}, M_J, M'_J }
+// (kCB x kCB each, row-major): X of L_JJ X = I, L_JJ X = L_{J,J-1} and
+// L_JJ^T X = L_{J+1,J}^T.  Rows past N act as identity rows.  The first also
+// writes dinv[i] = 1 / d_i.  A substitution goes row by row: lane = column,
+// warp w holds rows w, w + 8, ... in registers, and the row that is final
+// reaches the others through shared memory.  (FP64 instructions bound it: a
+// sub-partition issues a fourth of a block's 496 row updates, where one warp
+// with a column a lane issued all of them and the products of L_JJ^{-1} with
+// the off-diagonal blocks came on top: 50 us for any N, now 15.)
 __global__ void __launch_bounds__(256) k_coarse_prep(int N, int m, const double* __restrict__ Lc,
                                                      double* blk, double* dinv) {
   __shared__ double Lj[kCB][kCB + 1];
-  __shared__ double Li[kCB][kCB + 1];
-  __shared__ double Lo[kCB][kCB + 1];
-  const int J = blockIdx.x, NB = gridDim.x, base = J * kCB, tid = threadIdx.x;
-  double* out = blk + (long long)J * kCBlocks * kCB * kCB;
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-    const int r = e / kCB, q = e % kCB;
-    Lj[r][q] = q == r ? 1.0 : lower_at(Lc, N, m, base + r, base + q);
+  __shared__ double R[kCB][kCB + 1];           // right-hand sides in
+  __shared__ double row[2][kCB];
+  const int J = blockIdx.x, what = blockIdx.y, NB = gridDim.x, base = J * kCB, tid = threadIdx.x;
+  const int c = tid & 31, w = tid >> 5;
+  for (int e = tid; e < kCB * kCB; e += 256) {
+    // consecutive threads take consecutive rows: a band column is contiguous
+    const int r = e % kCB, q = e / kCB;
+    Lj[r][q] = lower_at(Lc, N, m, base + r, base + q);
+    if (what == 0) R[r][q] = r == q ? 1.0 : 0.0;
+    if (what == 1) R[r][q] = J > 0 ? lower_at(Lc, N, m, base + r, base - kCB + q) : 0.0;
+    if (what == 2) R[q][r] = J + 1 < NB ? lower_at(Lc, N, m, base + kCB + r, base + q) : 0.0;
   }
-  if (tid < kCB && base + tid < N) dinv[base + tid] = 1.0 / Lc[(long long)(base + tid) * (m + 1)];
+  if (what == 0 && tid < kCB && base + tid < N)
+    dinv[base + tid] = 1.0 / Lc[(long long)(base + tid) * (m + 1)];
   __syncthreads();
-  // inverse of the unit lower block, one column per thread (forward substitution)
-  if (tid < kCB) {
-    const int c = tid;
-    for (int r = 0; r < kCB; ++r) {
-      double s = r == c ? 1.0 : 0.0;
-      if (r > c) {
-        for (int q = c; q < r; ++q) s -= Lj[r][q] * Li[q][c];
-      }
-      Li[r][c] = s;
+  double x[kCB / 8];
+#pragma unroll
+  for (int k = 0; k < kCB / 8; ++k) x[k] = R[w + 8 * k][c];
+  const bool up = what == 2;                   // L^T: from the last row up
+#pragma unroll 8
+  for (int st = 0; st < kCB - 1; ++st) {
+    const int r = up ? kCB - 1 - st : st;
+    if (w == (r & 7)) {
+      double v = x[0];
+#pragma unroll
+      for (int k = 1; k < kCB / 8; ++k)
+        if ((r >> 3) == k) v = x[k];
+      row[st & 1][c] = v;
+    }
+    __syncthreads();
+    const double v = row[st & 1][c];
+#pragma unroll
+    for (int k = 0; k < kCB / 8; ++k) {
+      const int i = w + 8 * k;
+      if (up ? i < r : i > r) x[k] -= (up ? Lj[r][i] : Lj[i][r]) * v;   // uniform in a warp
     }
   }
-  __syncthreads();
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) out[e] = Li[e / kCB][e % kCB];
-  // M_J = L_JJ^{-1} L_{J,J-1}
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-    const int r = e / kCB, q = e % kCB;
-    Lo[r][q] = J > 0 ? lower_at(Lc, N, m, base + r, base - kCB + q) : 0.0;
-  }
-  __syncthreads();
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-    const int r = e / kCB, q = e % kCB;
-    double s = 0.0;
-    for (int k = 0; k < kCB; ++k) s += Li[r][k] * Lo[k][q];
-    out[kCB * kCB + e] = s;
-  }
-  __syncthreads();
-  // M'_J = L_JJ^{-T} L_{J+1,J}^T :  M'[c][q] = sum_k Li[k][c] L[(J+1)B + q][JB + k]
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-    const int q = e / kCB, kk = e % kCB;
-    Lo[q][kk] = J + 1 < NB ? lower_at(Lc, N, m, base + kCB + q, base + kk) : 0.0;
-  }
-  __syncthreads();
-  for (int e = tid; e < kCB * kCB; e += blockDim.x) {
-    const int c = e / kCB, q = e % kCB;
-    double s = 0.0;
-    for (int kk = 0; kk < kCB; ++kk) s += Li[kk][c] * Lo[q][kk];
-    out[2 * kCB * kCB + e] = s;
-  }
+  double* out = blk + ((long long)J * kCBlocks + what) * kCB * kCB;
+#pragma unroll
+  for (int k = 0; k < kCB / 8; ++k) out[(w + 8 * k) * kCB + c] = x[k];
 }
 
 __device__ __forceinline__ unsigned cl_rank() {
@@ -980,24 +1001,18 @@ __device__ __forceinline__ unsigned cl_rank() {
 __device__ __forceinline__ void cl_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// store v into the same shared-memory location of every CTA of the cluster
-__device__ __forceinline__ void cl_broadcast(const double* local, double v) {
+// store v into the same shared-memory location of CTA rk of the cluster
+__device__ __forceinline__ void cl_store(const double* local, int rk, double v) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(local);
-#pragma unroll
-  for (int rk = 0; rk < kCC; ++rk) {
-    unsigned ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rk));
-    asm volatile("st.relaxed.cluster.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
-  }
+  unsigned ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rk));
+  asm volatile("st.relaxed.cluster.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
 }
-__device__ __forceinline__ void cl_broadcast(const float* local, float v) {
+__device__ __forceinline__ void cl_store(const float* local, int rk, float v) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(local);
-#pragma unroll
-  for (int rk = 0; rk < kCC; ++rk) {
-    unsigned ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rk));
-    asm volatile("st.relaxed.cluster.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
-  }
+  unsigned ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rk));
+  asm volatile("st.relaxed.cluster.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
 }
 __device__ __forceinline__ unsigned long long ld_cl(const double* p) {
   unsigned long long v;
@@ -1086,79 +1101,108 @@ __global__ void __launch_bounds__(256, 1) k_coarse_solve_cluster(
   // ---- forward: L y = b ----
   for (int J = rank; J < NB; J += kCC) {
     const int base = J * kCB, row = base + r;
-    T acc = (h == 0 && row < N) ? T(rc[row]) : T(0);
-    for (int I = J - W > 0 ? J - W : 0; I <= J - 2; ++I) {
-      T yv[4] = {0.0, 0.0, 0.0, 0.0};
-      ok = ok && wait4(y + I * kCB + 4 * h, yv, abort_flag, status);
+    // everything that does not wait for another block is loaded first: the
+    // entries of L_JI one block ahead, the blocks' rows for the whole step
+    const T* Li = blk + (long long)J * kCBlocks * kCB * kCB;
+    const int I0 = J - W > 0 ? J - W : 0;
+    T li[4], mj[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      li[k] = Li[r * kCB + 4 * h + k];
+      mj[k] = J > 0 ? Li[kCB * kCB + r * kCB + 4 * h + k] : T(0);
+    }
+    auto load_l = [&](int I) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int c = I * kCB + 4 * h + k;
-        const T l = (row < N && row - c <= m) ? Lr[(long long)row * (m + 1) + (row - c)] : 0.0;
-        acc -= l * yv[k];
+        l[k] = (row < N && row - c <= m) ? Lr[(long long)row * (m + 1) + (row - c)] : T(0);
       }
+    };
+    if (I0 <= J - 2) load_l(I0);
+    T acc = (h == 0 && row < N) ? T(rc[row]) : T(0);
+    for (int I = I0; I <= J - 2; ++I) {
+      T lc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) lc[k] = l[k];
+      if (I < J - 2) load_l(I + 1);
+      T yv[4] = {0.0, 0.0, 0.0, 0.0};
+      ok = ok && wait4(y + I * kCB + 4 * h, yv, abort_flag, status);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc -= lc[k] * yv[k];
     }
     acc = sum8(acc);
     if (h == 0) uv[r] = acc;
     __syncthreads();
-    const T* Li = blk + (long long)J * kCBlocks * kCB * kCB;
     T s = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s += Li[r * kCB + 4 * h + k] * uv[4 * h + k];
+    for (int k = 0; k < 4; ++k) s += li[k] * uv[4 * h + k];
     s = sum8(s);
     if (J > 0) {
-      const T* M = Li + kCB * kCB;
       T yv[4] = {0.0, 0.0, 0.0, 0.0};
       ok = ok && wait4(y + (J - 1) * kCB + 4 * h, yv, abort_flag, status);
       T t = 0.0;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) t += M[r * kCB + 4 * h + k] * yv[k];
+      for (int k = 0; k < 4; ++k) t += mj[k] * yv[k];
       s -= sum8(t);
     }
-    __syncthreads();
-    if (h == 0) cl_broadcast(y + row, ok ? s : 0.0);
+    cl_store(y + row, h, ok ? s : T(0));       // lane h of a row to CTA h
+    __syncthreads();                           // uv is free again
   }
   // ---- backward: L^T x = D^{-1} y ----
   const int lastJ = NB - 1 - ((NB - 1 - rank) % kCC + kCC) % kCC;
   for (int I = lastJ; I >= 0; I -= kCC) {
     const int base = I * kCB, col = base + r;
+    const T* Li = blk + (long long)I * kCBlocks * kCB * kCB;
+    const int J0 = I + W < NB - 1 ? I + W : NB - 1;
+    T li[4], mt[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      li[k] = Li[(4 * h + k) * kCB + r];
+      mt[k] = I + 1 < NB ? Li[2 * kCB * kCB + r * kCB + 4 * h + k] : T(0);
+    }
+    auto load_l = [&](int J) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int rw = J * kCB + 4 * h + k;
+        l[k] = (rw < N && col < N && rw - col <= m) ? Lc[(long long)col * (m + 1) + (rw - col)] : T(0);
+      }
+    };
+    if (J0 >= I + 2) load_l(J0);
+    const T di = col < N ? dinv[col] : T(0);
     T acc = 0.0;
     if (h == 0) {
       T yv[4] = {0.0, 0.0, 0.0, 0.0};
       ok = ok && wait4(y + base + (r & ~3), yv, abort_flag, status);
-      acc = col < N ? yv[r & 3] * dinv[col] : 0.0;
+      acc = col < N ? yv[r & 3] * di : T(0);
     }
-    for (int J = I + W < NB - 1 ? I + W : NB - 1; J >= I + 2; --J) {
+    for (int J = J0; J >= I + 2; --J) {
+      T lc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) lc[k] = l[k];
+      if (J > I + 2) load_l(J - 1);
       T xv[4] = {0.0, 0.0, 0.0, 0.0};
       ok = ok && wait4(x + J * kCB + 4 * h, xv, abort_flag, status);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int rw = J * kCB + 4 * h + k;
-        const T l = (rw < N && col < N && rw - col <= m) ? Lc[(long long)col * (m + 1) + (rw - col)] : 0.0;
-        acc -= l * xv[k];
-      }
+      for (int k = 0; k < 4; ++k) acc -= lc[k] * xv[k];
     }
     acc = sum8(acc);
     if (h == 0) uv[r] = acc;
     __syncthreads();
-    const T* Li = blk + (long long)I * kCBlocks * kCB * kCB;
     T s = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s += Li[(4 * h + k) * kCB + r] * uv[4 * h + k];
+    for (int k = 0; k < 4; ++k) s += li[k] * uv[4 * h + k];
     s = sum8(s);
     if (I + 1 < NB) {
-      const T* Mt = Li + 2 * kCB * kCB;
       T xv[4] = {0.0, 0.0, 0.0, 0.0};
       ok = ok && wait4(x + (I + 1) * kCB + 4 * h, xv, abort_flag, status);
       T t = 0.0;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) t += Mt[r * kCB + 4 * h + k] * xv[k];
+      for (int k = 0; k < 4; ++k) t += mt[k] * xv[k];
       s -= sum8(t);
     }
+    cl_store(x + col, h, ok ? s : T(0));
+    if (h == 0 && col < N) pc[col] = s;
     __syncthreads();
-    if (h == 0) {
-      cl_broadcast(x + col, ok ? s : 0.0);
-      if (col < N) pc[col] = s;
-    }
   }
   cl_sync();   // no CTA leaves while others may still store into its shared memory
 }
@@ -1410,7 +1454,7 @@ __global__ void __launch_bounds__(256) k_band_lu_solve(int N, int m, const doubl
 template <class TP, class TR>
 __global__ void __launch_bounds__(256) k_restrict_fe_local(Geo g, CGeo c, const TP* __restrict__ P,
                                                            const TR* __restrict__ r, double* part) {
-  __shared__ double sh[8 * 32];
+  __shared__ double sh[8 * 8];
   const int ndx = c.nc[0] + 1, ndy = c.nc[1] + 1;
   const int D = blockIdx.x;
   const int j[3] = {D % ndx, (D / ndx) % ndy, D / (ndx * ndy)};
@@ -1466,7 +1510,7 @@ __global__ void k_restrict_fe_gather(CGeo c, const double* __restrict__ part, co
 // MSFV restriction: block sums of r.
 __global__ void __launch_bounds__(256) k_restrict_fv(Geo g, CGeo c, const double* __restrict__ r,
                                                      const int* __restrict__ perm, double* rc) {
-  __shared__ double sh[32];
+  __shared__ double sh[8];
   const int I = blockIdx.x;
   const int Ic[3] = {I % c.nc[0], (I / c.nc[0]) % c.nc[1], I / (c.nc[0] * c.nc[1])};
   const int bx = c.b[0], by = c.b[1], bz = c.b[2];
@@ -1560,9 +1604,9 @@ cudaError_t launch_galerkin_fe(const Geo& g, const CGeo& c, bool single, bool no
   }
   const int nd = (c.nc[0] + 1) * (c.nc[1] + 1) * (c.nc[2] + 1);
   if (single)
-    k_galerkin_fe_local<float><<<nd, 256, 0, s>>>(g, c, b.f32.P, b.Ad, b.Ax, b.Ay, b.Az, b.loc);
+    k_galerkin_fe_local<float><<<nd, block_threads(c), 0, s>>>(g, c, b.f32.P, b.Ad, b.Ax, b.Ay, b.Az, b.loc);
   else
-    k_galerkin_fe_local<double><<<nd, 256, 0, s>>>(g, c, b.P, b.Ad, b.Ax, b.Ay, b.Az, b.loc);
+    k_galerkin_fe_local<double><<<nd, block_threads(c), 0, s>>>(g, c, b.P, b.Ad, b.Ax, b.Ay, b.Az, b.loc);
   count_launches(1);
   k_galerkin_fe_gather<<<(27 * c.Nc + 255) / 256, 256, 0, s>>>(c, b.loc, b.Acs); count_launches(1);
   return cudaGetLastError();
@@ -1708,7 +1752,7 @@ cudaError_t launch_band_factor(int Nc, int m, int sym, Buffers& b, cudaStream_t 
   if (e != cudaSuccess) return e;
   const long long n = (long long)Nc * (m + 1);
   k_ldlt_rows<<<(int)((n + 255) / 256), 256, 0, s>>>(Nc, m, b.Lc, b.Lr);
-  k_coarse_prep<<<(Nc + kCB - 1) / kCB, 256, 0, s>>>(Nc, m, b.Lc, b.cblk, b.cdinv);
+  k_coarse_prep<<<dim3((Nc + kCB - 1) / kCB, kCBlocks), 256, 0, s>>>(Nc, m, b.Lc, b.cblk, b.cdinv);
   count_launches(launches + 2);
   if (b.f32.Lc) {
     // FP32 copy of the factor for the mixed-precision substitution
@@ -1727,13 +1771,13 @@ cudaError_t launch_restrict(const Geo& g, const CGeo& c, int kind, const double*
   if (kind == 0) {
     const int nd = (c.nc[0] + 1) * (c.nc[1] + 1) * (c.nc[2] + 1);
     // mixed precision: the FP32 copy of the handle's residual (written with it)
-    if (single && r == b.r) k_restrict_fe_local<float, float><<<nd, 256, 0, s>>>(g, c, b.f32.P, b.f32.r, b.loc);
-    else if (single) k_restrict_fe_local<float, double><<<nd, 256, 0, s>>>(g, c, b.f32.P, r, b.loc);
-    else k_restrict_fe_local<double, double><<<nd, 256, 0, s>>>(g, c, b.P, r, b.loc);
+    if (single && r == b.r) k_restrict_fe_local<float, float><<<nd, block_threads(c), 0, s>>>(g, c, b.f32.P, b.f32.r, b.loc);
+    else if (single) k_restrict_fe_local<float, double><<<nd, block_threads(c), 0, s>>>(g, c, b.f32.P, r, b.loc);
+    else k_restrict_fe_local<double, double><<<nd, block_threads(c), 0, s>>>(g, c, b.P, r, b.loc);
     count_launches(1);
     k_restrict_fe_gather<<<(c.Nc + 127) / 128, 128, 0, s>>>(c, b.loc, b.perm, b.rc); count_launches(1);
   } else {
-    k_restrict_fv<<<c.Nc, 256, 0, s>>>(g, c, r, b.perm, b.rc); count_launches(1);
+    k_restrict_fv<<<c.Nc, block_threads(c), 0, s>>>(g, c, r, b.perm, b.rc); count_launches(1);
   }
   return cudaGetLastError();
 }
