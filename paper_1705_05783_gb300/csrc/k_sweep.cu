@@ -214,9 +214,11 @@ __device__ __forceinline__ void sweep_index(const Shape& s, int x, int y, int z,
 // transposes: one CTA per (tile, kXC positions along x).  Rows are read or
 // written in the natural layout by warps along x (coalesced); records are
 // written or read by warps whose lanes are the tile's lanes, one chunk each;
-// shared memory holds the block in between.
+// shared memory holds the block in between.  FP64 takes 32 positions a CTA: the
+// FP64 unit bounds the residual there, and with 64 a grid of 500k cells gave
+// some SMs three CTAs of work and others two (19.5 against 18.4 us).
 template <class T>
-constexpr int kXC = 64;
+constexpr int kXC = sizeof(T) == 8 ? 32 : 64;
 // row stride of that block: in a record, lane ty + 1 sits one row down and one
 // chunk to the left; this stride keeps the chunks of a record on different banks
 template <class T>
@@ -284,14 +286,25 @@ __global__ void __launch_bounds__(256) k_resid_scaled(Geo g, Shape s, const T* _
       T v = T(0);                            // the tail of the row's last chunk
       if (y < g.ny && z < g.nz && x < g.nx) {
         const long long i = x + g.sy * y + g.sz * z;
-        T a = bv[i] - Ad[i] * xv[i];
-        if (x > 0) a -= Ax[i] * xv[i - 1];
-        if (x < g.nx - 1) a -= (kNS ? Axu : Ax)[i + 1] * xv[i + 1];
-        if (y > 0) a -= Ay[i] * xv[i - g.sy];
-        if (y < g.ny - 1) a -= (kNS ? Ayu : Ay)[i + g.sy] * xv[i + g.sy];
-        if (z > 0) a -= Az[i] * xv[i - g.sz];
-        if (z < g.nz - 1) a -= (kNS ? Azu : Az)[i + g.sz] * xv[i + g.sz];
-        v = a * dinv[i];
+        // every load before the first use, with a zero in place of a
+        // neighbour outside the grid (0 * 0 changes no sum): behind branches
+        // each neighbour's loads waited for the ones before
+        const bool xl = x > 0, xu = x < g.nx - 1, yl = y > 0, yu = y < g.ny - 1, zl = z > 0, zu = z < g.nz - 1;
+        const T cb = bv[i], cd = Ad[i], xc = xv[i], di = dinv[i];
+        const T c0 = xl ? Ax[i] : T(0), v0 = xl ? xv[i - 1] : T(0);
+        const T c1 = xu ? (kNS ? Axu : Ax)[i + 1] : T(0), v1 = xu ? xv[i + 1] : T(0);
+        const T c2 = yl ? Ay[i] : T(0), v2 = yl ? xv[i - g.sy] : T(0);
+        const T c3 = yu ? (kNS ? Ayu : Ay)[i + g.sy] : T(0), v3 = yu ? xv[i + g.sy] : T(0);
+        const T c4 = zl ? Az[i] : T(0), v4 = zl ? xv[i - g.sz] : T(0);
+        const T c5 = zu ? (kNS ? Azu : Az)[i + g.sz] : T(0), v5 = zu ? xv[i + g.sz] : T(0);
+        T a = cb - cd * xc;
+        a -= c0 * v0;
+        a -= c1 * v1;
+        a -= c2 * v2;
+        a -= c3 * v3;
+        a -= c4 * v4;
+        a -= c5 * v5;
+        v = a * di;
       }
       blk[r][h] = v;
     }
