@@ -37,6 +37,9 @@ struct cams_handle {
   int lev_grid[4] = {0, 0, 0, 0};
   bool lev_blocked[4] = {false, false, false, false};
   long long lev_lstride[4] = {0, 0, 0, 0};
+  // the basis solves in panels: widest band of the level (-1: not used), grid, scratch
+  int lev_pm[4] = {-1, -1, -1, -1}, lev_pgrid[4] = {0, 0, 0, 0};
+  long long lev_pstride[4] = {0, 0, 0, 0};
   long long lev_gbytes[4] = {0, 0, 0, 0};   // > 0: the level's windows in b.lwork, bytes per CTA
   long long lwork_len = 0;
   long long lscratch_len = 0;
@@ -352,8 +355,8 @@ int alloc_all(cams_handle* h) {
       return fail(h, CAMS_ECUDA, "cudaMemset failed");
   }
   AL(b.red, kColBlocks);
-  AL(b.tick, 1);
-  if (cudaMemset(b.tick, 0, sizeof(unsigned)) != cudaSuccess)
+  AL(b.tick, 2);
+  if (cudaMemset(b.tick, 0, 2 * sizeof(unsigned)) != cudaSuccess)
     return fail(h, CAMS_ECUDA, "cudaMemset failed");
   AL(b.scal, 8);
   AL(b.status, 1);
@@ -675,6 +678,12 @@ int update_operators(cams_handle* h, int force, int* n_rebuilt) {
       if (lev == 3 && h->surr_tol > 0.0 && h->surr_n > 0 && rebuilt == ne) {
         const int rc = surrogate_interiors(h);
         if (rc) return rc;
+      }
+      if (h->lev_pm[lev] >= 0) {
+        CK(launch_entity_panel(h->g, b.ents + f, b.flag + f, h->lev_count[lev], h->lev_pm[lev],
+                               h->lev_pgrid[lev], h->lev_pstride[lev], adaptive ? 1 : 0, h->single, b,
+                               h->stream));
+        continue;
       }
       CK(launch_entity_solve(h->g, b.ents + f, b.flag + f, h->lev_count[lev], h->lev_smem[lev],
                              h->lev_grid[lev], h->lev_lstride[lev], adaptive ? 1 : 0, h->single,
@@ -1055,6 +1064,23 @@ int cams_setup(const cams_grid* grid, const cams_fluid* fluid, const cams_option
     }
     h->lev_smem[lev] = sm;
     h->lev_lstride[lev] = ls;
+    // the basis functions are solved in panels where the ring of columns fits
+    // (k_basis_panel.cu; in FP64 from half-width 16 on, where the panels win)
+    const int threads = entity_panel_threads(mmax), psm = entity_panel_smem(mmax, h->single);
+    const bool use = h->single || mmax >= 16;
+    if (h->lev_count[lev] > 0 && use && threads > 0 && psm + 1024 <= (int)prop.sharedMemPerBlockOptin) {
+      if (set_entity_panel_smem(mmax, h->single) != cudaSuccess) {
+        delete h;
+        return fail(nullptr, CAMS_ECUDA, "cudaFuncSetAttribute failed");
+      }
+      const int per_sm = std::min((int)prop.sharedMemPerMultiprocessor / (psm + 2048), 2048 / threads);
+      h->lev_pm[lev] = mmax;
+      h->lev_pgrid[lev] = std::min(h->lev_count[lev], prop.multiProcessorCount * std::max(1, per_sm));
+      for (int e = h->lev_first[lev]; e < h->lev_first[lev] + h->lev_count[lev]; ++e)
+        h->lev_pstride[lev] = std::max(h->lev_pstride[lev], entity_panel_scratch(h->ents[e]));
+      const long long len = h->lev_pgrid[lev] * h->lev_pstride[lev];
+      h->lscratch_len = std::max(h->lscratch_len, h->single ? (len + 1) / 2 : len);
+    }
     if (h->lev_blocked[lev] && sm > (int)prop.sharedMemPerBlockOptin) {
       // the blocked solver's window in global memory (the 15^3 interiors of
       // 16^3 blocks): per CTA the same bytes, 256-byte aligned

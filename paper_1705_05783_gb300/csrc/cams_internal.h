@@ -140,7 +140,7 @@ struct Buffers {
   double* r = nullptr;                                    // residual (natural order)
   double* cf = nullptr;                                   // correction function Psi (N; FP64 with options.cf)
   double* red = nullptr;                                  // reduction partials
-  unsigned* tick = nullptr;                               // CTAs that have left theirs
+  unsigned* tick = nullptr;                               // CTAs that have left theirs; the next entity
   double* scal = nullptr;                                 // reduced scalars (device)
   int* status = nullptr;                                  // device status word
   SingleBuffers f32;                                      // mixed precision only
@@ -210,6 +210,16 @@ cudaError_t launch_entity_solve(const Geo& g, const Entity* ents, const unsigned
                                 bool single, bool blocked, long long gbytes, Buffers& b,
                                 cudaStream_t s);
 int entity_smem_bytes(const Entity& E, bool single, bool blocked);
+// The basis solves in panels (k_basis_panel.cu) of a level whose widest band
+// is m: threads of a CTA (0: too wide), shared memory, scratch elements of one
+// entity.
+int entity_panel_threads(int m);
+int entity_panel_smem(int m, bool single);
+long long entity_panel_scratch(const Entity& E);
+cudaError_t set_entity_panel_smem(int m, bool single);
+cudaError_t launch_entity_panel(const Geo& g, const Entity* ents, const unsigned char* flag, int count,
+                                int m, int grid, long long lstride, int adaptive, bool single,
+                                Buffers& b, cudaStream_t s);
 cudaError_t launch_entity_cf(const Geo& g, const Entity* ents, int count, int smem, int grid,
                              long long lstride, bool single, bool blocked, long long gbytes,
                              Buffers& b, cudaStream_t s);

@@ -14,62 +14,21 @@
 // local solve and P are FP64, or FP32 for the mixed-precision preconditioner
 // (the basis operator is read in FP64 and rounded).
 //
+// The basis functions of most levels are solved in panels instead
+// (k_basis_panel.cu); these kernels keep narrow FP64 bands, windows too wide
+// for that kernel's shared memory, and the correction functions.
+//
 // The same kernels in their kCF form apply the correction functions of
 // Table 1 step 4 (Sec. 3): the same local systems with one right-hand side,
 // the fine residual r minus the couplings to the correction values Psi
 // already found on the lower levels (zero on the vertices), launched level
 // by level like the basis stages.
 #include "cams_internal.h"
+#include "entity.h"
 
 namespace cams {
 
 namespace {
-
-__device__ __forceinline__ double coupling(const Geo& g, const double* Abx, const double* Aby,
-                                           const double* Abz, int d, long long i) {
-  // A_b entry between i and i - e_d (stored at the upper cell)
-  return d == 0 ? Abx[i] : (d == 1 ? Aby[i] : Abz[i]);
-}
-
-__device__ __forceinline__ long long gstride(const Geo& g, int d) {
-  return d == 0 ? 1 : (d == 1 ? g.sy : g.sz);
-}
-
-__device__ __forceinline__ int gextent(const Geo& g, int d) {
-  return d == 0 ? g.nx : (d == 1 ? g.ny : g.nz);
-}
-
-// global slot (bits over x,y,z) of the entity's r-th right-hand side
-__device__ __forceinline__ int slot_of(int r, int free_mask) {
-  int s = 0, k = 0;
-  for (int d = 0; d < 3; ++d)
-    if (free_mask & (1 << d)) {
-      if (r & (1 << k)) s |= 1 << d;
-      ++k;
-    }
-  return s;
-}
-
-struct Local {
-  int c[3];        // coordinates
-  long long i;     // global cell
-};
-
-__device__ __forceinline__ Local local_cell(const Entity& E, int l) {
-  Local L;
-  const int L0 = E.L[E.ord[0]], L1 = E.L[E.ord[1]];
-  int t[3];
-  t[0] = l % L0;
-  t[1] = (l / L0) % L1;
-  t[2] = l / (L0 * L1);
-  for (int k = 0; k < 3; ++k) L.c[E.ord[k]] = E.org[E.ord[k]] + t[k];
-  return L;
-}
-
-__device__ __forceinline__ int local_stride(const Entity& E, int d) {
-  const int L0 = E.L[E.ord[0]], L1 = E.L[E.ord[1]];
-  return d == E.ord[0] ? 1 : (d == E.ord[1] ? L0 : L0 * L1);
-}
 
 // Build row l of M (lower band, ring slot) and the right-hand sides of row l:
 // one per corner vertex for the basis functions, or (kCF) the single
@@ -251,15 +210,7 @@ __global__ void __launch_bounds__(256) k_entity_solve(
       }
       for (int s = 0; s < 8; ++s) P[(long long)s * g.N + i] = T(0);
       for (int r = 0; r < nr; ++r) P[(long long)slot_of(r, E.free_mask) * g.N + i] = Y[l * nr + r];
-      if (adaptive) {
-        snap[0 * g.N + i] = Abd[i];
-        snap[1 * g.N + i] = c.c[0] > 0 ? Abx[i] : 0.0;
-        snap[2 * g.N + i] = c.c[0] < g.nx - 1 ? Abx[i + 1] : 0.0;
-        snap[3 * g.N + i] = c.c[1] > 0 ? Aby[i] : 0.0;
-        snap[4 * g.N + i] = c.c[1] < g.ny - 1 ? Aby[i + g.sy] : 0.0;
-        snap[5 * g.N + i] = c.c[2] > 0 ? Abz[i] : 0.0;
-        snap[6 * g.N + i] = c.c[2] < g.nz - 1 ? Abz[i + g.sz] : 0.0;
-      }
+      if (adaptive) snapshot_row(g, c, i, Abd, Abx, Aby, Abz, snap);
     }
     __syncthreads();
   }
@@ -581,15 +532,7 @@ __global__ void __launch_bounds__(256) k_entity_solve_blk(
       }
       for (int s = 0; s < 8; ++s) P[(long long)s * g.N + i] = T(0);
       for (int r = 0; r < nr; ++r) P[(long long)slot_of(r, E.free_mask) * g.N + i] = Y[l * nr + r];
-      if (adaptive) {
-        snap[0 * g.N + i] = Abd[i];
-        snap[1 * g.N + i] = c.c[0] > 0 ? Abx[i] : 0.0;
-        snap[2 * g.N + i] = c.c[0] < g.nx - 1 ? Abx[i + 1] : 0.0;
-        snap[3 * g.N + i] = c.c[1] > 0 ? Aby[i] : 0.0;
-        snap[4 * g.N + i] = c.c[1] < g.ny - 1 ? Aby[i + g.sy] : 0.0;
-        snap[5 * g.N + i] = c.c[2] > 0 ? Abz[i] : 0.0;
-        snap[6 * g.N + i] = c.c[2] < g.nz - 1 ? Abz[i + g.sz] : 0.0;
-      }
+      if (adaptive) snapshot_row(g, c, i, Abd, Abx, Aby, Abz, snap);
     }
     __syncthreads();
   }
