@@ -65,6 +65,7 @@ struct cams_handle {
   bool ilu_pipelined = true;    // false: level-scheduled sweeps (CAMS_ILU_LEVEL=1)
   bool ilu_cta = false;         // blocks of tiles per cluster, else every tile on its own
   bool coarse_cluster = false;  // MSFE coarse solve across a cluster (CAMS_COARSE_CLUSTER=0: one CTA)
+  Twist twist;                  // the two-ended factorisation that goes with the cluster solve (H = 0: none)
   bool coarse_inv = false;      // mixed MSFE: FP32 factor and inverse factor (CAMS_COARSE_INV=0: off)
   // learned surrogate of the interior basis stage (cams_set_surrogate)
   double surr_tol = 0.0;           // > 0: enabled
@@ -280,6 +281,12 @@ void build_entities(cams_handle* h, std::vector<int>& ent_of_cell) {
   }
 }
 
+// rows of a coarse band, and elements of the (one or two) coarse bands
+size_t coarse_rows(const cams_handle* h) { return h->twist.H > 0 ? h->twist.Ns : h->c.Nc; }
+size_t coarse_len(const cams_handle* h) {
+  return (h->twist.H > 0 ? 2 : 1) * coarse_rows(h) * (size_t)(h->mc + 1);
+}
+
 int alloc_all(cams_handle* h) {
   const long long N = h->g.N;
   Buffers& b = h->b;
@@ -310,8 +317,8 @@ int alloc_all(cams_handle* h) {
       f.Axu = f.Ax; f.Ayu = f.Ay; f.Azu = f.Az;
     }
     AL(f.P, 8 * N); AL(f.pc, h->c.Nc);
-    AL(f.Lc, (size_t)h->c.Nc * (h->mc + 1)); AL(f.Lr, (size_t)h->c.Nc * (h->mc + 1));
-    AL(f.cblk, coarse_blocks_len(h->c.Nc)); AL(f.cdinv, h->c.Nc);
+    AL(f.Lc, coarse_len(h)); AL(f.Lr, coarse_len(h));
+    AL(f.cblk, 2 * coarse_blocks_len(coarse_rows(h))); AL(f.cdinv, 2 * coarse_rows(h));
     if (h->coarse_inv) {
       AL(f.Z, (size_t)h->c.Nc * (size_t)coarse_ldz(h->c.Nc));
       AL(f.tc, coarse_ldz(h->c.Nc));
@@ -330,10 +337,10 @@ int alloc_all(cams_handle* h) {
   if (h->lwork_len > 0) AL(b.lwork, (size_t)h->lwork_len);
   AL(b.loc, (size_t)h->n_dual * 36);
   AL(b.Acs, 27LL * h->c.Nc);
-  AL(b.band, (size_t)h->c.Nc * (2 * h->mc + 1));
+  AL(b.band, std::max((size_t)h->c.Nc * (2 * h->mc + 1), coarse_len(h)));
   AL(b.Fc, (size_t)h->c.Nc * (2 * h->mc + 1));
-  AL(b.Lc, (size_t)h->c.Nc * (h->mc + 1)); AL(b.Lr, (size_t)h->c.Nc * (h->mc + 1));
-  AL(b.cblk, coarse_blocks_len(h->c.Nc)); AL(b.cdinv, h->c.Nc); AL(b.cabort, 1);
+  AL(b.Lc, coarse_len(h)); AL(b.Lr, coarse_len(h));
+  AL(b.cblk, 2 * coarse_blocks_len(coarse_rows(h))); AL(b.cdinv, 2 * coarse_rows(h)); AL(b.cabort, 1);
   AL(b.perm, h->c.Nc);
   AL(b.jxt, 2LL * h->g.nx);
   AL(b.rc, h->c.Nc); AL(b.pc, h->c.Nc); AL(b.ywork, h->c.Nc);
@@ -704,6 +711,7 @@ int update_operators(cams_handle* h, int force, int* n_rebuilt) {
     // MSFE with a symmetric A: R A P = P^T A P is symmetric (LDL^T), else band LU
     const int sym = o.restriction != 1 && !nonsym;
     h->coarse_ldlt = sym != 0;
+    b.twist = h->coarse_cluster ? h->twist : Twist();
     if (h->coarse_inv) {
       CK(launch_coarse_factor_inv(h->c, h->mc, b, h->stream));
     } else {
@@ -1124,6 +1132,12 @@ int cams_setup(const cams_grid* grid, const cams_fluid* fluid, const cams_option
     const char* ci = std::getenv("CAMS_COARSE_INV");
     h->coarse_inv = h->single && opt->restriction != 1 && !opt->jacobian &&
                     !(ci && ci[0] == '0') && coarse_inverse_ok(c.Nc, h->mc);
+    // R A P is symmetric, and stays what the last build made it (restriction 2
+    // overwrites it with its closing MSFV operator)
+    const Twist tw = coarse_twist(c.Nc, h->mc);
+    if (opt->restriction == 0 && !opt->jacobian && !h->coarse_inv &&
+        coarse_twist_ok(tw, (int)prop.sharedMemPerBlockOptin))
+      h->twist = tw;
   }
   rc = alloc_all(h);
   if (rc) {
@@ -1273,6 +1287,14 @@ int cams_set_schedule(cams_handle* h, int ilu_cta, int coarse_cluster) {
   CK(cudaStreamSynchronize(h->stream));
   if (ilu_cta >= 0) h->ilu_cta = ilu_cta == 1;
   if (coarse_cluster >= 0) h->coarse_cluster = coarse_cluster == 1;
+  const Twist tw = h->coarse_cluster ? h->twist : Twist();
+  if (h->coarse_ldlt && !h->coarse_inv && tw.H != h->b.twist.H) {
+    // the solve changes kernels: factor the current R A P in the layout it reads
+    h->b.twist = tw;
+    CK(cudaMemsetAsync(h->b.Lc, 0, sizeof(double) * coarse_len(h), h->stream));
+    CK(launch_band_fill(h->c, h->mc, 1, h->b, h->stream));
+    CK(launch_band_factor(h->c.Nc, h->mc, 1, h->b, h->stream));
+  }
   if (h->step_exec) {                          // it holds the previous schedule's kernels
     CK(cudaGraphExecDestroy(h->step_exec));
     h->step_exec = nullptr;
@@ -1706,6 +1728,19 @@ int cams_get(cams_handle* h, int what, double* dst) {
     case CAMS_Q_COARSE: CK(cudaMemcpyAsync(dst, b.Acs, sizeof(double) * 27 * h->c.Nc, k, s)); break;
     case CAMS_Q_COARSE_FACTOR:
       if (!h->coarse_ldlt) return fail(h, CAMS_EINVAL, "the coarse matrix was not factored by L D L^T");
+      if (b.twist.H > 0) {
+        // the handle's factor is of the two-ended order: form the one asked for
+        const size_t len = (size_t)h->c.Nc * (h->mc + 1);
+        double* tmp = nullptr;
+        CK(cudaMalloc(&tmp, 2 * len * sizeof(double)));
+        cudaError_t e = cudaMemsetAsync(tmp, 0, 2 * len * sizeof(double), s);
+        if (e == cudaSuccess) e = launch_ldlt_plain(h->c, h->mc, b, tmp, tmp + len, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, tmp + len, sizeof(double) * len, k, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        cudaFree(tmp);
+        CK(e);
+        break;
+      }
       CK(cudaMemcpyAsync(dst, b.Lc, sizeof(double) * h->c.Nc * (h->mc + 1), k, s));
       break;
     case CAMS_Q_ILU_DIAG: {

@@ -43,6 +43,17 @@ struct CGeo {
   int Nc;
 };
 
+// The band factorisation of the coarse matrix from both ends (k_coarse.cu):
+// H rows at either end, mm in the middle, Ns = H + mm rows in each of the two
+// bands, which follow one another in memory.  H = 0: one band, in order.
+struct Twist {
+  int H = 0, mm = 0, Ns = 0;
+#ifdef __CUDACC__
+  __host__ __device__
+#endif
+  long long stride(int m) const { return (long long)Ns * (m + 1); }
+};
+
 // One local entity of the wirebasket: an edge segment (level 1), face patch
 // (level 2) or dual-block interior (level 3).  It is the box of cells
 // [org, org + L) where every lattice (non-free) direction has L = 1.
@@ -127,6 +138,7 @@ struct Buffers {
   double *Lc = nullptr, *Lr = nullptr;                    // LDL^T factor, column/row-major
   double *cblk = nullptr, *cdinv = nullptr;               // block inverses / products, 1/d
   int* cabort = nullptr;                                  // abort flag of the cluster solve
+  Twist twist;                                            // how band, Lc, Lr, cblk, cdinv are laid out
   int* perm = nullptr;                                    // coarse natural -> band order
   int* jxt = nullptr;                                     // per x: the two coarse x-corners (-1: none)
   double *rc = nullptr, *pc = nullptr;                    // coarse vectors (band order)
@@ -250,6 +262,11 @@ cudaError_t launch_band_solve(int Nc, int m, int sym, bool cluster, bool single,
                               cudaStream_t s);
 long long coarse_blocks_len(int Nc);
 bool coarse_cluster_ok(int Nc, int max_smem);
+Twist coarse_twist(int Nc, int m);
+bool coarse_twist_ok(const Twist& tw, int max_smem);
+// L D L^T of R A P in band order, whatever layout the handle's own factor has
+// (band, Lc: Nc (m + 1) elements each)
+cudaError_t launch_ldlt_plain(const CGeo& c, int m, Buffers& b, double* band, double* Lc, cudaStream_t s);
 // FP64: p += P p_c; single: delta = P p_c (FP32 P and delta)
 cudaError_t launch_prolong_add(const Geo& g, const CGeo& c, bool single, Buffers& b,
                                cudaStream_t s);

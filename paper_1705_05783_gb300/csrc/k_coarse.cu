@@ -369,9 +369,11 @@ __global__ void __launch_bounds__(128) k_galerkin_fe_ns(
 
 // Natural-order 27-point stencil -> column-major band in the reordered
 // index.  General (MSFV): Bc[col*(2m+1) + (row - col + m)].  Symmetric
-// (MSFE): lower triangle only, W[col*(m+1) + (row - col)].
+// (MSFE): lower triangle only, W[col*(m+1) + (row - col)].  With tw.H > 0 the
+// rows from the end, beyond the first tw.Ns, go to the second band with the
+// order reversed (see Twist).
 template <class TB>
-__global__ void k_band_fill(CGeo c, int m, int sym, const double* __restrict__ Acs,
+__global__ void k_band_fill(CGeo c, int m, int sym, Twist tw, const double* __restrict__ Acs,
                             const int* __restrict__ perm, TB* band) {
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (q >= 27LL * c.Nc) return;
@@ -387,7 +389,11 @@ __global__ void k_band_fill(CGeo c, int m, int sym, const double* __restrict__ A
   }
   const int row = perm[I], col = perm[J];
   if (sym) {
-    if (row >= col) band[(long long)col * (m + 1) + (row - col)] = (TB)Acs[q];
+    if (row < col) return;
+    if (tw.H > 0 && row >= tw.Ns)
+      band[tw.stride(m) + (long long)(c.Nc - 1 - row) * (m + 1) + (row - col)] = (TB)Acs[q];
+    else
+      band[(long long)col * (m + 1) + (row - col)] = (TB)Acs[q];
   } else {
     band[(long long)col * (2 * m + 1) + (row - col + m)] = (TB)Acs[q];
   }
@@ -442,8 +448,13 @@ __device__ __forceinline__ T band_at(const T* W, int m, int r, int c) {
 // T: the precision of the factorisation (FP64, or FP32 for the mixed
 // preconditioner's coarse solve)
 template <class T>
-__global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, const T* __restrict__ Wr,
-                                                    T* W, T* Lc, int* status) {
+__global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long long stride,
+                                                    const T* __restrict__ Wr, T* W, T* Lc,
+                                                    int* status) {
+  // blockIdx.y: which of the two bands of a twisted factorisation
+  Wr += blockIdx.y * stride;
+  W += blockIdx.y * stride;
+  Lc += blockIdx.y * stride;
   __shared__ T A[kTB][kTB + 1];        // diagonal block; column q keeps d_q l_rq
   __shared__ T L[kTB][kTB + 1];        // l_rq below the diagonal
   __shared__ T rinv[kTB];              // 1 / d_q
@@ -575,10 +586,31 @@ __global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, const 
     Lc[(long long)c0 * (m + 1) + tid] = tid == 0 ? A[0][0] : L[tid][0];
 }
 
+// ---- the twisted factorisation ----
+// The block steps of a band L D L^T depend on one another, and a step takes
+// about 10 us whatever the band holds (a launch, the loads, 16 pivots).  So
+// the band is eliminated from both ends at once: the first H rows in order,
+// the last H in reverse order (the second band, whose row l is the matrix's
+// row N - 1 - l), both up to the mm = N - 2 H rows in the middle.  Each band has
+// Ns = H + mm rows; the second's middle starts as zeros and ends as what its
+// elimination subtracts there, which is added to the first's before the middle
+// is eliminated.  (N - mm) / 32 + mm / 16 steps instead of N / 16, and the
+// substitutions go the same two ways (k_coarse_solve_twisted).
+// Lattice workload 32x8x8 (N = 2048, m = 73), FP64: factorisation 1.30 -> 0.71 ms.
+__global__ void k_twist_merge(Twist tw, int m, double* W) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int j = (int)(e / (m + 1)), d = (int)(e % (m + 1)), i = j + d;   // middle entry (i, j)
+  if (i >= tw.mm) return;
+  W[(long long)(tw.H + j) * (m + 1) + d] +=
+      W[tw.stride(m) + (long long)(tw.H + tw.mm - 1 - i) * (m + 1) + d];
+}
+
 // Row-major copy of L for the backward substitution: Lr[k*(m+1) + a] = l_{k,k-a}.
-__global__ void k_ldlt_rows(int N, int m, const double* __restrict__ Lc, double* Lr) {
+__global__ void k_ldlt_rows(int N, int m, long long stride, const double* __restrict__ Lc, double* Lr) {
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (e >= (long long)N * (m + 1)) return;
+  Lc += blockIdx.y * stride;
+  Lr += blockIdx.y * stride;
   const int k = (int)(e / (m + 1)), a = (int)(e % (m + 1));
   Lr[e] = (a == 0) ? Lc[(long long)k * (m + 1)] : (k - a >= 0 ? Lc[(long long)(k - a) * (m + 1) + a] : 0.0);
 }
@@ -948,8 +980,17 @@ __device__ __forceinline__ double lower_at(const double* Lc, int N, int m, int r
 // sub-partition issues a fourth of a block's 496 row updates, where one warp
 // with a column a lane issued all of them and the products of L_JJ^{-1} with
 // the off-diagonal blocks came on top: 50 us for any N, now 15.)
-__global__ void __launch_bounds__(256) k_coarse_prep(int N, int m, const double* __restrict__ Lc,
-                                                     double* blk, double* dinv) {
+// blockIdx.z: which band of a twisted factorisation; the second one's blocks
+// end at row H.
+__global__ void __launch_bounds__(256) k_coarse_prep(int N, int m, int H, long long stride,
+                                                     const double* __restrict__ Lc, double* blk,
+                                                     double* dinv) {
+  if (blockIdx.z == 1) {
+    if ((int)blockIdx.x * kCB >= H) return;
+    Lc += stride;
+    blk += (long long)gridDim.x * kCBlocks * kCB * kCB;
+    dinv += N;
+  }
   __shared__ double Lj[kCB][kCB + 1];
   __shared__ double R[kCB][kCB + 1];           // right-hand sides in
   __shared__ double row[2][kCB];
@@ -1202,6 +1243,160 @@ __global__ void __launch_bounds__(256, 1) k_coarse_solve_cluster(
     }
     cl_store(x + col, h, ok ? s : T(0));
     if (h == 0 && col < N) pc[col] = s;
+    __syncthreads();
+  }
+  cl_sync();   // no CTA leaves while others may still store into its shared memory
+}
+
+// The same across the two bands of a twisted factorisation: four CTAs take
+// the blocks of the first band, four those of the second, each up to the
+// middle, whose rows (first band) also take the second band's products; on
+// the way back the middle's values reach the second band in its reversed
+// order.  y and x are kept for both bands in every CTA (Np each; the rows past
+// the second band's end read as zero).  1000 unknowns, half-width 111, FP64:
+// 69 -> 53 us a solve.
+constexpr int kTG = kCC / 2;                 // CTAs of a band
+
+template <class T>
+__global__ void __launch_bounds__(256, 1) k_coarse_solve_twisted(
+    int N, int m, Twist tw, const T* __restrict__ Lc, const T* __restrict__ Lr,
+    const T* __restrict__ blk, const T* __restrict__ dinv, const double* __restrict__ rc, T* pc,
+    int* abort_flag, int* status) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  T* sm = reinterpret_cast<T*>(sm_raw);
+  __shared__ T uv[kCB];
+  const int Ns = tw.Ns, H = tw.H, NB = (Ns + kCB - 1) / kCB, HB = H / kCB, Np = NB * kCB;
+  const int rank = (int)cl_rank(), side = rank / kTG, first = rank % kTG;
+  T* const y = sm + side * Np;
+  T* const x = sm + (2 + side) * Np;
+  const T* const yB = sm + Np;               // the second band's
+  T* const xB = sm + 3 * Np;
+  const T* const LrB = Lr + tw.stride(m);
+  Lc += side * tw.stride(m);
+  Lr += side * tw.stride(m);
+  blk += (long long)side * NB * kCBlocks * kCB * kCB;
+  dinv += side * Ns;
+  const int tid = threadIdx.x, r = tid >> 3, h = tid & 7;
+  const int W = (m + kCB - 1) / kCB;
+  for (int i = tid; i < 4 * Np; i += blockDim.x)
+    sm[i] = i >= 3 * Np + Ns ? T(0) : CWord<T>::value(CWord<T>::kNR);
+  cl_sync();
+  bool ok = true;
+  // ---- forward ----
+  const int fend = side == 0 ? NB : HB;
+  for (int J = first; J < fend; J += kTG) {
+    const int base = J * kCB, row = base + r;
+    const T* Li = blk + (long long)J * kCBlocks * kCB * kCB;
+    const int I0 = J - W > 0 ? J - W : 0;
+    T li[4], mj[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      li[k] = Li[r * kCB + 4 * h + k];
+      mj[k] = J > 0 ? Li[kCB * kCB + r * kCB + 4 * h + k] : T(0);
+    }
+    auto load_l = [&](const T* L, int rw, int I) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = I * kCB + 4 * h + k;
+        l[k] = (row < Ns && rw - c <= m) ? L[(long long)rw * (m + 1) + (rw - c)] : T(0);
+      }
+    };
+    T acc = (h == 0 && row < Ns) ? T(rc[side == 0 ? row : N - 1 - row]) : T(0);
+    if (J >= HB) {                           // the middle: the second band's part
+      const int rb = Ns - 1 - (row - H);
+      for (int I = HB - W > 0 ? HB - W : 0; I < HB; ++I) {
+        load_l(LrB, rb, I);
+        T yv[4] = {0.0, 0.0, 0.0, 0.0};
+        ok = ok && wait4(yB + I * kCB + 4 * h, yv, abort_flag, status);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc -= l[k] * yv[k];
+      }
+    }
+    if (I0 <= J - 2) load_l(Lr, row, I0);
+    for (int I = I0; I <= J - 2; ++I) {
+      T lc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) lc[k] = l[k];
+      if (I < J - 2) load_l(Lr, row, I + 1);
+      T yv[4] = {0.0, 0.0, 0.0, 0.0};
+      ok = ok && wait4(y + I * kCB + 4 * h, yv, abort_flag, status);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc -= lc[k] * yv[k];
+    }
+    acc = sum8(acc);
+    if (h == 0) uv[r] = acc;
+    __syncthreads();
+    T s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += li[k] * uv[4 * h + k];
+    s = sum8(s);
+    if (J > 0) {
+      T yv[4] = {0.0, 0.0, 0.0, 0.0};
+      ok = ok && wait4(y + (J - 1) * kCB + 4 * h, yv, abort_flag, status);
+      T t = 0.0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t += mj[k] * yv[k];
+      s -= sum8(t);
+    }
+    cl_store(y + row, h, ok ? s : T(0));
+    __syncthreads();
+  }
+  // ---- backward ----
+  const int last = fend - 1 - ((fend - 1 - first) % kTG + kTG) % kTG;
+  for (int I = last; I >= 0; I -= kTG) {
+    const int base = I * kCB, col = base + r;
+    const T* Li = blk + (long long)I * kCBlocks * kCB * kCB;
+    const int J0 = I + W < NB - 1 ? I + W : NB - 1;
+    T li[4], mt[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      li[k] = Li[(4 * h + k) * kCB + r];
+      mt[k] = I + 1 < NB ? Li[2 * kCB * kCB + r * kCB + 4 * h + k] : T(0);
+    }
+    auto load_l = [&](int J) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int rw = J * kCB + 4 * h + k;
+        l[k] = (rw < Ns && col < Ns && rw - col <= m) ? Lc[(long long)col * (m + 1) + (rw - col)] : T(0);
+      }
+    };
+    if (J0 >= I + 2) load_l(J0);
+    const T di = col < Ns ? dinv[col] : T(0);
+    T acc = 0.0;
+    if (h == 0) {
+      T yv[4] = {0.0, 0.0, 0.0, 0.0};
+      ok = ok && wait4(y + base + (r & ~3), yv, abort_flag, status);
+      acc = col < Ns ? yv[r & 3] * di : T(0);
+    }
+    for (int J = J0; J >= I + 2; --J) {
+      T lc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) lc[k] = l[k];
+      if (J > I + 2) load_l(J - 1);
+      T xv[4] = {0.0, 0.0, 0.0, 0.0};
+      ok = ok && wait4(x + J * kCB + 4 * h, xv, abort_flag, status);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc -= lc[k] * xv[k];
+    }
+    acc = sum8(acc);
+    if (h == 0) uv[r] = acc;
+    __syncthreads();
+    T s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += li[k] * uv[4 * h + k];
+    s = sum8(s);
+    if (I + 1 < NB) {
+      T xv[4] = {0.0, 0.0, 0.0, 0.0};
+      ok = ok && wait4(x + (I + 1) * kCB + 4 * h, xv, abort_flag, status);
+      T t = 0.0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t += mt[k] * xv[k];
+      s -= sum8(t);
+    }
+    const T out = ok ? s : T(0);
+    cl_store(x + col, h, out);
+    if (I >= HB && col < Ns) cl_store(xB + (Ns - 1 - (col - H)), h, out);   // (the first band's CTAs)
+    if (h == 0 && col < Ns) pc[side == 0 ? col : N - 1 - col] = s;
     __syncthreads();
   }
   cl_sync();   // no CTA leaves while others may still store into its shared memory
@@ -1626,10 +1821,12 @@ cudaError_t launch_galerkin_fv(const Geo& g, const CGeo& c, bool single, bool no
 }
 
 cudaError_t launch_band_fill(const CGeo& c, int m, int sym, Buffers& b, cudaStream_t s) {
-  const size_t len = sym ? (size_t)c.Nc * (m + 1) : (size_t)c.Nc * (2 * m + 1);
+  const Twist tw = sym ? b.twist : Twist();
+  const size_t len = tw.H > 0 ? (size_t)(2 * tw.stride(m))
+                              : (sym ? (size_t)c.Nc * (m + 1) : (size_t)c.Nc * (2 * m + 1));
   cudaError_t e = cudaMemsetAsync(b.band, 0, sizeof(double) * len, s);
   if (e != cudaSuccess) return e;
-  k_band_fill<double><<<(27 * c.Nc + 255) / 256, 256, 0, s>>>(c, m, sym, b.Acs, b.perm, b.band);
+  k_band_fill<double><<<(27 * c.Nc + 255) / 256, 256, 0, s>>>(c, m, sym, tw, b.Acs, b.perm, b.band);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1637,30 +1834,68 @@ cudaError_t launch_band_fill(const CGeo& c, int m, int sym, Buffers& b, cudaStre
 // The symmetric band factorisation: one launch per block of kTB columns,
 // each allowed to start while the previous one drains (programmatic
 // dependent launch; the kernel waits for its predecessor).
+// (columns [from, to) of `bands` bands of N rows)
 template <class T>
-static cudaError_t ldlt_launches(int Nc, int m, T* band, T* Lc, int* status, cudaStream_t s,
-                                 int& launches) {
+static cudaError_t ldlt_launches(int N, int m, int from, int to, int bands, long long stride, T* band,
+                                 T* Lc, int* status, cudaStream_t s, int& launches) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  for (int c0 = 0; c0 < Nc; c0 += kTB) {
-    const int c1 = (c0 + kTB < Nc ? c0 + kTB : Nc) - 1;
-    const int rhi = (c1 + m < Nc - 1) ? c1 + m : Nc - 1;
+  for (int c0 = from; c0 < to; c0 += kTB) {
+    const int c1 = (c0 + kTB < N ? c0 + kTB : N) - 1;
+    const int rhi = (c1 + m < N - 1) ? c1 + m : N - 1;
     const int nb = rhi > c1 ? (rhi - c1 - 1 + kTB) / kTB : 0;
     const int grid = nb > 0 ? nb * (nb + 1) / 2 : 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(grid, bands);
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = c0 == 0 ? 0 : 1;      // the first block follows the band fill normally
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_ldlt_block<T>, Nc, m, c0, (const T*)band, band, Lc,
-                                       status);
+    cfg.numAttrs = c0 == from ? 0 : 1;   // the first block follows the kernel before it normally
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_ldlt_block<T>, N, m, c0, stride, (const T*)band, band,
+                                       Lc, status);
     if (e != cudaSuccess) return e;
     ++launches;
   }
   return cudaSuccess;
+}
+
+// The two ends' rows are whole blocks of the substitution; a middle of at
+// least m rows keeps them apart.  Below two blocks an end there is little to
+// gain (12 x 12 x 4 coarse nodes gain, 8 x 8 lattices are one launch chain of 4).
+Twist coarse_twist(int Nc, int m) {
+  Twist tw;
+  const int H = Nc > m ? kCB * ((Nc - m) / (2 * kCB)) : 0;
+  if (H < 2 * kCB) return tw;
+  tw.H = H;
+  tw.mm = Nc - 2 * H;
+  tw.Ns = H + tw.mm;
+  return tw;
+}
+
+static cudaError_t ldlt_factor(int Nc, int m, const Twist& tw, double* band, double* Lc, int* status,
+                               cudaStream_t s, int& launches) {
+  if (tw.H == 0) return ldlt_launches<double>(Nc, m, 0, Nc, 1, 0, band, Lc, status, s, launches);
+  const long long st = tw.stride(m);
+  cudaError_t e = ldlt_launches<double>(tw.Ns, m, 0, tw.H, 2, st, band, Lc, status, s, launches);
+  if (e != cudaSuccess) return e;
+  const long long n = (long long)tw.mm * (m + 1);
+  k_twist_merge<<<(int)((n + 255) / 256), 256, 0, s>>>(tw, m, band);
+  ++launches;
+  return ldlt_launches<double>(tw.Ns, m, tw.H, tw.Ns, 1, st, band, Lc, status, s, launches);
+}
+
+cudaError_t launch_ldlt_plain(const CGeo& c, int m, Buffers& b, double* band, double* Lc,
+                              cudaStream_t s) {
+  Buffers t = b;
+  t.twist = Twist();
+  t.band = band;
+  cudaError_t e = launch_band_fill(c, m, 1, t, s);
+  int launches = 0;
+  if (e == cudaSuccess) e = ldlt_factor(c.Nc, m, t.twist, band, Lc, b.status, s, launches);
+  count_launches(launches);
+  return e;
 }
 
 long long coarse_ldz(int Nc) { return ((long long)Nc + kZS - 1) / kZS * kZS; }
@@ -1692,7 +1927,7 @@ cudaError_t launch_coarse_factor_inv(const CGeo& c, int m, Buffers& b, cudaStrea
   cudaError_t e = launch_band_fill(c, m, 1, b, s);
   if (e != cudaSuccess) return e;
   int launches = 0;
-  e = ldlt_launches<double>(Nc, m, b.band, b.Lc, b.status, s, launches);
+  e = ldlt_factor(Nc, m, Twist(), b.band, b.Lc, b.status, s, launches);
   if (e != cudaSuccess) return e;
   const long long n = (long long)Nc * (m + 1);
   k_to_single<<<(int)((n + 255) / 256), 256, 0, s>>>((int)n, b.Lc, b.f32.Lc);
@@ -1748,19 +1983,21 @@ cudaError_t launch_band_factor(int Nc, int m, int sym, Buffers& b, cudaStream_t 
     count_launches(launches);
     return cudaGetLastError();
   }
-  cudaError_t e = ldlt_launches<double>(Nc, m, b.band, b.Lc, b.status, s, launches);
+  const Twist& tw = b.twist;
+  cudaError_t e = ldlt_factor(Nc, m, tw, b.band, b.Lc, b.status, s, launches);
   if (e != cudaSuccess) return e;
-  const long long n = (long long)Nc * (m + 1);
-  k_ldlt_rows<<<(int)((n + 255) / 256), 256, 0, s>>>(Nc, m, b.Lc, b.Lr);
-  k_coarse_prep<<<dim3((Nc + kCB - 1) / kCB, kCBlocks), 256, 0, s>>>(Nc, m, b.Lc, b.cblk, b.cdinv);
+  const int bands = tw.H > 0 ? 2 : 1, N = tw.H > 0 ? tw.Ns : Nc, blocks = (N + kCB - 1) / kCB;
+  const long long n = (long long)N * (m + 1);
+  k_ldlt_rows<<<dim3((unsigned)((n + 255) / 256), bands), 256, 0, s>>>(N, m, n, b.Lc, b.Lr);
+  k_coarse_prep<<<dim3(blocks, kCBlocks, bands), 256, 0, s>>>(N, m, tw.H, n, b.Lc, b.cblk, b.cdinv);
   count_launches(launches + 2);
   if (b.f32.Lc) {
     // FP32 copy of the factor for the mixed-precision substitution
-    const long long nb = coarse_blocks_len(Nc);
-    k_to_single<<<(int)((n + 255) / 256), 256, 0, s>>>((int)n, b.Lc, b.f32.Lc);
-    k_to_single<<<(int)((n + 255) / 256), 256, 0, s>>>((int)n, b.Lr, b.f32.Lr);
+    const long long nb = bands * coarse_blocks_len(N), n2 = bands * n;
+    k_to_single<<<(int)((n2 + 255) / 256), 256, 0, s>>>((int)n2, b.Lc, b.f32.Lc);
+    k_to_single<<<(int)((n2 + 255) / 256), 256, 0, s>>>((int)n2, b.Lr, b.f32.Lr);
     k_to_single<<<(int)((nb + 255) / 256), 256, 0, s>>>((int)nb, b.cblk, b.f32.cblk);
-    k_to_single<<<(Nc + 255) / 256, 256, 0, s>>>(Nc, b.cdinv, b.f32.cdinv);
+    k_to_single<<<(bands * N + 255) / 256, 256, 0, s>>>(bands * N, b.cdinv, b.f32.cdinv);
     count_launches(4);
   }
   return cudaGetLastError();
@@ -1797,6 +2034,15 @@ static int coarse_smem_optin() {
 
 static int coarse_cluster_smem(int Nc, int bytes = 8) {
   return bytes * 2 * ((Nc + kCB - 1) / kCB) * kCB;
+}
+static int coarse_twist_smem(const Twist& tw, int bytes = 8) {
+  return 2 * coarse_cluster_smem(tw.Ns, bytes);
+}
+
+bool coarse_twist_ok(const Twist& tw, int max_smem) {
+  return tw.H > 0 && coarse_twist_smem(tw) <= max_smem &&
+         raise_smem_limit(k_coarse_solve_twisted<double>, coarse_twist_smem(tw)) == cudaSuccess &&
+         raise_smem_limit(k_coarse_solve_twisted<float>, coarse_twist_smem(tw, 4)) == cudaSuccess;
 }
 
 bool coarse_cluster_ok(int Nc, int max_smem) {
@@ -1841,7 +2087,19 @@ cudaError_t launch_band_solve(int Nc, int m, int sym, bool cluster, bool single,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (single) {
+    const Twist& tw = b.twist;
+    if (tw.H > 0) {
+      const SingleBuffers& f = b.f32;
+      cfg.dynamicSmemBytes = (size_t)coarse_twist_smem(tw, single ? 4 : 8);
+      e = single ? cudaLaunchKernelEx(&cfg, k_coarse_solve_twisted<float>, Nc, m, tw,
+                                      (const float*)f.Lc, (const float*)f.Lr, (const float*)f.cblk,
+                                      (const float*)f.cdinv, (const double*)b.rc, b.f32.pc, b.cabort,
+                                      b.status)
+                 : cudaLaunchKernelEx(&cfg, k_coarse_solve_twisted<double>, Nc, m, tw,
+                                      (const double*)b.Lc, (const double*)b.Lr, (const double*)b.cblk,
+                                      (const double*)b.cdinv, (const double*)b.rc, b.pc, b.cabort,
+                                      b.status);
+    } else if (single) {
       // FP32 substitution with the FP64 factor's FP32 copy; the result goes
       // straight to the FP32 prolongation
       const SingleBuffers& f = b.f32;
