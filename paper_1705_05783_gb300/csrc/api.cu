@@ -320,9 +320,11 @@ int alloc_all(cams_handle* h) {
     AL(f.Lc, coarse_len(h)); AL(f.Lr, coarse_len(h));
     AL(f.cblk, 2 * coarse_blocks_len(coarse_rows(h))); AL(f.cdinv, 2 * coarse_rows(h));
     if (h->coarse_inv) {
-      AL(f.Z, (size_t)h->c.Nc * (size_t)coarse_ldz(h->c.Nc));
-      AL(f.tc, coarse_ldz(h->c.Nc));
-      AL(f.zpart, coarse_part_len(h->c.Nc));
+      const int n = (int)coarse_rows(h);
+      AL(f.Z, (size_t)(n + h->twist.H) * (size_t)coarse_ldz(n));
+      AL(f.tc, 2 * coarse_ldz(n));
+      AL(f.zpart, 2 * coarse_part_len(n));
+      AL(f.G, coarse_g_len(h->twist, h->mc));
     }
     AL(f.lo, 4 * S); AL(f.up, 4 * S); AL(f.z, S);
     // slots that hold no cell must read as zero (the sweeps run branch-free over them)
@@ -386,7 +388,7 @@ void free_all(cams_handle* h) {
   const SingleBuffers& f = b.f32;
   void* fptrs[] = {f.Ad, f.Ax, f.Ay, f.Az, f.dinv, f.lo, f.up,
                    f.z, f.d, f.r, f.P, f.pc, f.Qx, f.Qy, f.Qz, f.Lc, f.Lr, f.cblk, f.cdinv,
-                   f.Z, f.tc, f.zpart, f.Axu != f.Ax ? f.Axu : nullptr, f.Ayu != f.Ay ? f.Ayu : nullptr,
+                   f.Z, f.tc, f.zpart, f.G, f.Axu != f.Ax ? f.Axu : nullptr, f.Ayu != f.Ay ? f.Ayu : nullptr,
                    f.Azu != f.Az ? f.Azu : nullptr};
   for (void* p : fptrs)
     if (p) cudaFree(p);
@@ -711,7 +713,7 @@ int update_operators(cams_handle* h, int force, int* n_rebuilt) {
     // MSFE with a symmetric A: R A P = P^T A P is symmetric (LDL^T), else band LU
     const int sym = o.restriction != 1 && !nonsym;
     h->coarse_ldlt = sym != 0;
-    b.twist = h->coarse_cluster ? h->twist : Twist();
+    b.twist = h->coarse_cluster || h->coarse_inv ? h->twist : Twist();
     if (h->coarse_inv) {
       CK(launch_coarse_factor_inv(h->c, h->mc, b, h->stream));
     } else {
@@ -1135,8 +1137,9 @@ int cams_setup(const cams_grid* grid, const cams_fluid* fluid, const cams_option
     // R A P is symmetric, and stays what the last build made it (restriction 2
     // overwrites it with its closing MSFV operator)
     const Twist tw = coarse_twist(c.Nc, h->mc);
-    if (opt->restriction == 0 && !opt->jacobian && !h->coarse_inv &&
-        coarse_twist_ok(tw, (int)prop.sharedMemPerBlockOptin))
+    if (opt->restriction == 0 && !opt->jacobian &&
+        (h->coarse_inv ? coarse_twist_inv_ok(tw, h->mc)
+                       : coarse_twist_ok(tw, (int)prop.sharedMemPerBlockOptin)))
       h->twist = tw;
   }
   rc = alloc_all(h);

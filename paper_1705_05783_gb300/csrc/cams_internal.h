@@ -101,9 +101,10 @@ struct SingleBuffers {
   // FP32 copy of the symmetric coarse factor (the substitution's operands)
   float *Lc = nullptr, *Lr = nullptr, *cblk = nullptr, *cdinv = nullptr;
   // the inverse-factor coarse solve: Z = L^{-1} of the FP32 copy Lc of the
-  // FP64 factor (Nc x coarse_ldz(Nc), column-major), the partial sums of
-  // Z b and t = D^{-1} Z b
-  float *Z = nullptr, *tc = nullptr, *zpart = nullptr;
+  // FP64 factor (column-major, leading dimension coarse_ldz(rows); twisted: the
+  // first band's Ns columns, then the second's H), the partial sums of Z b,
+  // t = D^{-1} Z b, and the middle's coupling G of a twisted factorisation
+  float *Z = nullptr, *tc = nullptr, *zpart = nullptr, *G = nullptr;
 };
 
 // Device buffers, one allocation each, owned by the handle.
@@ -264,6 +265,8 @@ long long coarse_blocks_len(int Nc);
 bool coarse_cluster_ok(int Nc, int max_smem);
 Twist coarse_twist(int Nc, int m);
 bool coarse_twist_ok(const Twist& tw, int max_smem);
+bool coarse_twist_inv_ok(const Twist& tw, int m);
+long long coarse_g_len(const Twist& tw, int m);
 // L D L^T of R A P in band order, whatever layout the handle's own factor has
 // (band, Lc: Nc (m + 1) elements each)
 cudaError_t launch_ldlt_plain(const CGeo& c, int m, Buffers& b, double* band, double* Lc, cudaStream_t s);

@@ -404,7 +404,7 @@ __global__ void k_band_fill(CGeo c, int m, int sym, Twist tw, const double* __re
 // kTB x kTB diagonal block in shared memory (redundantly: cheaper than a
 // separate launch), forms the panel rows l_rq (q in the block) of the
 // kTB-row tiles it owns, and subtracts  sum_q l_rq d_q l_cq  from its tile of
-// the trailing band.  Diagonal-tile CTAs write their panel rows to the
+// the trailing band.  The CTAs of its first tile column write their rows to the
 // factor Lc (column-major: Lc[q*(m+1) + (r-q)], Lc[q*(m+1)] = d_q).  The
 // working band W is only read in the block columns and only written right of
 // them, so CTAs of one launch never race.
@@ -447,8 +447,13 @@ __device__ __forceinline__ T band_at(const T* W, int m, int r, int c) {
 
 // T: the precision of the factorisation (FP64, or FP32 for the mixed
 // preconditioner's coarse solve)
-template <class T>
-__global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long long stride,
+// KT: tiles of the trailing band a CTA updates, side by side in a row of tiles
+// (one panel of kTB rows more for each).  The diagonal block and the panels
+// keep an SM's FP64 units busy, so two CTAs on one SM take twice the time:
+// with more tiles than SMs a CTA takes two.  (Half-width 211, two bands, 210
+// tiles: 29.6 us a step with KT = 1, 13.1 with KT = 2; one band, 105 tiles, KT = 1: 10.8.)
+template <class T, int KT>
+__global__ void __launch_bounds__(192 + 64 * KT) k_ldlt_block(int N, int m, int c0, long long stride,
                                                     const T* __restrict__ Wr, T* W, T* Lc,
                                                     int* status) {
   // blockIdx.y: which of the two bands of a twisted factorisation
@@ -458,8 +463,9 @@ __global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long l
   __shared__ T A[kTB][kTB + 1];        // diagonal block; column q keeps d_q l_rq
   __shared__ T L[kTB][kTB + 1];        // l_rq below the diagonal
   __shared__ T rinv[kTB];              // 1 / d_q
-  __shared__ T V[2 * kTB][kTB + 1];    // panel rows: a_rq in, l_rq out
-  __shared__ T VD[2 * kTB][kTB + 1];   // d_q l_rq of the panel rows
+  constexpr int kP = 1 + KT;           // panels: my row of tiles, then my columns
+  __shared__ T V[kP * kTB][kTB + 1];   // panel rows: a_rq in, l_rq out
+  __shared__ T VD[kP * kTB][kTB + 1];  // d_q l_rq of the panel rows
   const int c1 = min(c0 + kTB, N) - 1;
   const int tb = c1 - c0 + 1;
   const int tid = threadIdx.x;
@@ -467,11 +473,11 @@ __global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long l
   const int rlo = c1 + 1;
   const int rhi = min(c1 + m, N - 1);
   const int nb = rhi >= rlo ? (rhi - rlo + kTB) / kTB : 0;
-  int bi = 0, bj = 0;
+  int bi = 0, bj = 0;                  // (bj: the first of my tiles)
   {
     int t = blockIdx.x;
-    while (t > bi) { t -= bi + 1; ++bi; }
-    bj = t;
+    while (t > bi / KT) { t -= bi / KT + 1; ++bi; }
+    bj = KT * t;
   }
   const bool have_tile = nb > 0 && bi < nb;
   const int r0 = rlo + bi * kTB, cc0 = rlo + bj * kTB;
@@ -480,15 +486,15 @@ __global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long l
   // visible (a no-op when launched without the attribute).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  // --- stage the diagonal block and the 2 kTB panel rows ---
+  // --- stage the diagonal block and the panel rows ---
   // (consecutive threads take consecutive rows of one band column: the
   // column is contiguous in the band)
-  {
+  if (tid < kTB * kTB) {
     const int r = tid % kTB, q = tid / kTB;
     A[r][q] = (r < tb && q <= r) ? band_at(Wr, m, c0 + r, c0 + q) : T(0);
   }
-  for (int e = tid; e < 2 * kTB * kTB; e += blockDim.x) {
-    const int k = e % (2 * kTB), q = e / (2 * kTB);
+  for (int e = tid; e < kP * kTB * kTB; e += blockDim.x) {
+    const int k = e % (kP * kTB), q = e / (kP * kTB);
     const int r = (k < kTB ? r0 + k : cc0 + k - kTB);
     V[k][q] = (have_tile && r <= rhi && q < tb) ? band_at(Wr, m, r, c0 + q) : T(0);
   }
@@ -509,7 +515,7 @@ __global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long l
     rinv[0] = pivot_rcp(A[0][0], bad);
     if (bad && blockIdx.x == 0) atomicOr(status, kStatSingular);
   }
-  // panel rows, four threads a row in warps 4-7
+  // panel rows, four threads a row from warp 4 on
   const int pk = (tid - 128) >> 2, pt = tid & 3;
   const int src0 = (threadIdx.x & 31) & ~3;
   T v[kTB / 4];
@@ -563,17 +569,20 @@ __global__ void __launch_bounds__(256) k_ldlt_block(int N, int m, int c0, long l
     for (int j = 0; j < kTB / 4; ++j) V[pk][4 * j + pt] = v[j];
   }
   __syncthreads();
-  if (have_tile) {
-    // W[r][c] -= sum_q l_rq d_q l_cq, one element a thread
+  if (have_tile && tid < kTB * kTB) {
+    // W[r][c] -= sum_q l_rq d_q l_cq, one element of a tile a thread
     const int a = tid / kTB, b = tid % kTB;
-    const int r = r0 + a, cc = cc0 + b;
-    if (r <= rhi && cc <= rhi && cc <= r && r - cc <= m) {
-      T s = T(0);
-      for (int q = 0; q < tb; ++q) s = fma(V[a][q], VD[kTB + b][q], s);
-      W[(long long)cc * (m + 1) + (r - cc)] -= s;
+#pragma unroll
+    for (int t = 0; t < KT; ++t) {
+      const int r = r0 + a, cc = cc0 + t * kTB + b;
+      if (r <= rhi && cc <= rhi && cc <= r && r - cc <= m) {
+        T s = T(0);
+        for (int q = 0; q < tb; ++q) s = fma(V[a][q], VD[(1 + t) * kTB + b][q], s);
+        W[(long long)cc * (m + 1) + (r - cc)] -= s;
+      }
     }
-    // diagonal tiles publish their panel rows
-    if (bi == bj) {
+    // CTAs of the first tile column publish their panel rows
+    if (bj == 0) {
       const int a2 = tid / kTB, q = tid % kTB;
       const int r2 = r0 + a2, col = c0 + q;
       if (r2 <= rhi && q < tb && r2 - col <= m) Lc[(long long)col * (m + 1) + (r2 - col)] = V[a2][q];
@@ -678,9 +687,17 @@ __device__ __forceinline__ void zband(float4& acc, const float* Lt, int kb, cons
   }
 }
 
-__global__ void __launch_bounds__(kZT, 1) k_coarse_zinv(int N, int m, int ring,
+// blockIdx.y = 1: the second band of a twisted factorisation, whose rows end at
+// H; its Z follows the first band's N columns.
+__global__ void __launch_bounds__(kZT, 1) k_coarse_zinv(int N, int m, int H, int ring,
                                                       const float* __restrict__ Lc, float* Z,
                                                       long long ldz) {
+  if (blockIdx.y == 1) {
+    Lc += (long long)N * (m + 1);
+    Z += N * ldz;
+    N = H;
+    if ((int)blockIdx.x * kZCols >= N) return;
+  }
   // [3][m + 32][32] band tiles, [2][kZQ - 1][kZG][32] float4 far sums,
   // [kZQ - 1][kZG][32] float4 near sums, [kZG][2 ring] float4 rings
   extern __shared__ __align__(16) float zsm[];
@@ -790,17 +807,26 @@ __global__ void __launch_bounds__(kZT, 1) k_coarse_zinv(int N, int m, int ring,
 // part[c * ldz + i].  b is the FP64 restricted residual, rounded to FP32.
 constexpr int kZS = 128;   // rows per strip
 constexpr int kZK = 256;   // columns per chunk
-__global__ void __launch_bounds__(256) k_coarse_zlower(int N, const float* __restrict__ Z,
-                                                       long long ldz, const double* __restrict__ rhs,
-                                                       float* part) {
+// Twisted (H > 0): blockIdx.z = 1 is the second band, of H rows in reverse order
+// from the end of the Nc; the first band's middle takes its own b only.
+__global__ void __launch_bounds__(256) k_coarse_zlower(int N, int Nc, int H,
+                                                       const float* __restrict__ Z, long long ldz,
+                                                       const double* __restrict__ rhs, float* part) {
+  const bool second = blockIdx.z == 1;
+  if (second) {
+    Z += N * ldz;
+    part += (long long)gridDim.y * ldz;
+    N = H;
+  }
   __shared__ float4 red[8][32];
   __shared__ float bs[kZK];                        // the chunk's b, rounded to FP32 once
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i0 = blockIdx.x * kZS, c = blockIdx.y, jc = c * kZK;
-  if (jc > i0 + kZS - 1 || jc >= N) return;        // the whole chunk lies above the strip
+  // the whole chunk lies above the strip, or the strip past the band's end
+  if (jc > i0 + kZS - 1 || jc >= N || i0 >= N) return;
   // (an FP64 -> FP32 conversion is an FP64-unit instruction: one per
   // element here, not one per element and warp in the loop below)
-  for (int e = threadIdx.x; e < kZK; e += blockDim.x) bs[e] = jc + e < N ? (float)rhs[jc + e] : 0.f;
+  for (int e = threadIdx.x; e < kZK; e += blockDim.x) bs[e] = jc + e < N ? (float)rhs[second ? Nc - 1 - (jc + e) : jc + e] : 0.f;
   __syncthreads();
   const int ib = i0 + 4 * lane;                    // my rows ib .. ib + 3
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -840,12 +866,131 @@ __global__ void k_coarse_tsum(int N, int m, const float* __restrict__ Lc,
   t[i] = s / Lc[(long long)i * (m + 1)];
 }
 
+// The twisted form, N = H + mm rows in the first band: t of both bands,
+// y_i = (Z b)_i as above.  With C the second band's entries of L in the middle
+// rows (its last mb = min(m, H) columns) and Z_mm the middle's block of Z,
+// G = -Z_mm C (k_coarse_g) carries the middle's part both ways:
+//   y_mid += G y_b,  t_mid = y_mid / d,  t_b = y_b / d + G^T t_mid,
+// so that x = Z^T t needs no further step for the second band.  CTA 0 takes
+// the middle and the second band's last mb rows, the others the rest.
+constexpr int kMidMax = 512;    // rows of the middle
+constexpr int kMidT = 1024;
+__global__ void __launch_bounds__(kMidT) k_coarse_tsum2(int N, int m, int H,
+                                                        const float* __restrict__ Lc,
+                                                        const float* __restrict__ G, int ldg,
+                                                        const float* __restrict__ part,
+                                                        long long ldz, int chunks, float* t) {
+  const int mm = N - H, mb = min(m, H), tid = threadIdx.x;
+  const float* const Lb = Lc + (long long)N * (m + 1);
+  const float* const pb = part + (long long)chunks * ldz;
+  auto total = [&](const float* p, int i) {
+    float s = 0.f;
+    const int n = i / kZK + 1;
+#pragma unroll 8
+    for (int c = 0; c < n; ++c) s += p[(long long)c * ldz + i];
+    return s;
+  };
+  if (blockIdx.x > 0) {
+    const int i = (blockIdx.x - 1) * kMidT + tid;      // H rows of the first, H - mb of the second
+    if (i < H) t[i] = total(part, i) / Lc[(long long)i * (m + 1)];
+    else if (i < 2 * H - mb) t[ldz + i - H] = total(pb, i - H) / Lb[(long long)(i - H) * (m + 1)];
+    return;
+  }
+  __shared__ float yb[kMidMax], tm[kMidMax], red[kMidT];
+  float ym = 0.f;
+  if (tid < kMidMax) {
+    if (tid < mm) ym = total(part, H + tid);
+  } else if (tid - kMidMax < mb) {
+    yb[tid - kMidMax] = total(pb, H - mb + tid - kMidMax);
+  }
+  __syncthreads();
+  {
+    const int groups = kMidT / ldg, grp = tid / ldg, i = tid % ldg;
+    float s = 0.f;
+    if (grp < groups && i < mm) {
+#pragma unroll 16
+      for (int c = grp; c < mb; c += groups) s = fmaf(G[(long long)c * ldg + i], yb[c], s);
+    }
+    red[tid] = s;
+    __syncthreads();
+    if (tid < mm) {
+      for (int q = 0; q < groups; ++q) ym += red[q * ldg + tid];
+      const float v = ym / Lc[(long long)(H + tid) * (m + 1)];
+      tm[tid] = v;
+      t[H + tid] = v;
+    }
+  }
+  __syncthreads();
+  // four columns a warp at a time, so that their loads overlap
+  constexpr int kW = kMidT / 32;
+  for (int c = tid >> 5; c < mb; c += 4 * kW) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int i = tid & 31; i < mm; i += 32) {
+      const float v = tm[i];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (c + k * kW < mb) s[k] = fmaf(G[(long long)(c + k * kW) * ldg + i], v, s[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+      const int cc = c + k * kW;
+      if ((tid & 31) == 0 && cc < mb)
+        t[ldz + H - mb + cc] = yb[cc] / Lb[(long long)(H - mb + cc) * (m + 1)] + s[k];
+    }
+  }
+}
+
+// G = -Z_mm C, four columns a CTA, one row a thread; column c of C is nonzero
+// in the middle rows j >= mm - 1 - (m - mb + c).
+__global__ void __launch_bounds__(kMidMax) k_coarse_g(int N, int m, int H, const float* __restrict__ Lc,
+                                                      const float* __restrict__ Z, long long ldz,
+                                                      float* G, int ldg) {
+  __shared__ float4 C[kMidMax];
+  const int mm = N - H, mb = min(m, H), c0 = 4 * blockIdx.x, i = threadIdx.x;
+  const float* const Lb = Lc + (long long)N * (m + 1);
+  if (i < mm) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = c0 + k, d = mm - 1 - i + mb - c;   // the second band's row H + mm - 1 - i
+      v[k] = c < mb && d <= m ? Lb[(long long)(H - mb + c) * (m + 1) + d] : 0.f;
+    }
+    C[i] = make_float4(v[0], v[1], v[2], v[3]);
+  }
+  __syncthreads();
+  if (i >= mm) return;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  const int jlo = max(0, mm - 1 - (m - mb + c0 + 3));
+#pragma unroll 8
+  for (int j = jlo; j <= i; ++j) {
+    const float z = Z[(long long)(H + j) * ldz + H + i];
+    const float4 cj = C[j];
+    s[0] = fmaf(-z, cj.x, s[0]);
+    s[1] = fmaf(-z, cj.y, s[1]);
+    s[2] = fmaf(-z, cj.z, s[2]);
+    s[3] = fmaf(-z, cj.w, s[3]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (c0 + k < mb) G[(long long)(c0 + k) * ldg + i] = s[k];
+}
+
 // x = Z^T t: one warp per column j (its rows i >= j are contiguous), 16-byte
 // loads from the aligned row j & ~3 on.
-__global__ void __launch_bounds__(256) k_coarse_zupper(int N, const float* __restrict__ Z,
-                                                       long long ldz, const float* __restrict__ t,
-                                                       float* x) {
+// (blockIdx.y = 1: the second band of a twisted factorisation, as in k_coarse_zlower)
+__global__ void __launch_bounds__(256) k_coarse_zupper(int N, int Nc, int H,
+                                                       const float* __restrict__ Z, long long ldz,
+                                                       const float* __restrict__ t, float* x) {
   const int lane = threadIdx.x & 31;
+  const bool second = blockIdx.y == 1;
+  if (second) {
+    Z += N * ldz;
+    t += ldz;
+    N = H;
+  }
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (j >= N) return;
   const float* col = Z + (long long)j * ldz;
@@ -861,7 +1006,7 @@ __global__ void __launch_bounds__(256) k_coarse_zupper(int N, const float* __res
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) x[j] = acc;
+  if (lane == 0) x[second ? Nc - 1 - j : j] = acc;
 }
 
 // L D L^T x = b, one CTA.  y lives in shared memory; the factor is streamed
@@ -1834,6 +1979,15 @@ cudaError_t launch_band_fill(const CGeo& c, int m, int sym, Buffers& b, cudaStre
 // The symmetric band factorisation: one launch per block of kTB columns,
 // each allowed to start while the previous one drains (programmatic
 // dependent launch; the kernel waits for its predecessor).
+// CTAs of a step with nb x nb tiles (lower triangle), kt tiles a CTA, and the
+// number that the chip runs one an SM
+constexpr int kLdltCtas = 152;
+static int ldlt_ctas(int nb, int kt) {
+  int n = 0;
+  for (int i = 0; i < nb; ++i) n += i / kt + 1;
+  return n;
+}
+
 // (columns [from, to) of `bands` bands of N rows)
 template <class T>
 static cudaError_t ldlt_launches(int N, int m, int from, int to, int bands, long long stride, T* band,
@@ -1845,16 +1999,17 @@ static cudaError_t ldlt_launches(int N, int m, int from, int to, int bands, long
     const int c1 = (c0 + kTB < N ? c0 + kTB : N) - 1;
     const int rhi = (c1 + m < N - 1) ? c1 + m : N - 1;
     const int nb = rhi > c1 ? (rhi - c1 - 1 + kTB) / kTB : 0;
-    const int grid = nb > 0 ? nb * (nb + 1) / 2 : 1;
+    const int kt = bands * ldlt_ctas(nb, 1) > kLdltCtas ? 2 : 1;
+    const int grid = nb > 0 ? ldlt_ctas(nb, kt) : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, bands);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(192 + 64 * kt);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = c0 == from ? 0 : 1;   // the first block follows the kernel before it normally
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_ldlt_block<T>, N, m, c0, stride, (const T*)band, band,
-                                       Lc, status);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kt == 2 ? k_ldlt_block<T, 2> : k_ldlt_block<T, 1>, N, m,
+                                       c0, stride, (const T*)band, band, Lc, status);
     if (e != cudaSuccess) return e;
     ++launches;
   }
@@ -1867,7 +2022,7 @@ static cudaError_t ldlt_launches(int N, int m, int from, int to, int bands, long
 Twist coarse_twist(int Nc, int m) {
   Twist tw;
   const int H = Nc > m ? kCB * ((Nc - m) / (2 * kCB)) : 0;
-  if (H < 2 * kCB) return tw;
+  if (H < 2 * kCB || 2 * ldlt_ctas((m + kTB - 1) / kTB, 2) > kLdltCtas) return tw;
   tw.H = H;
   tw.mm = Nc - 2 * H;
   tw.Ns = H + tw.mm;
@@ -1927,31 +2082,55 @@ cudaError_t launch_coarse_factor_inv(const CGeo& c, int m, Buffers& b, cudaStrea
   cudaError_t e = launch_band_fill(c, m, 1, b, s);
   if (e != cudaSuccess) return e;
   int launches = 0;
-  e = ldlt_factor(Nc, m, Twist(), b.band, b.Lc, b.status, s, launches);
+  e = ldlt_factor(Nc, m, b.twist, b.band, b.Lc, b.status, s, launches);
   if (e != cudaSuccess) return e;
-  const long long n = (long long)Nc * (m + 1);
+  const long long n = b.twist.H > 0 ? 2 * b.twist.stride(m) : (long long)Nc * (m + 1);
   k_to_single<<<(int)((n + 255) / 256), 256, 0, s>>>((int)n, b.Lc, b.f32.Lc);
   count_launches(launches + 1);
   return cudaGetLastError();
 }
 
+// The twisted form keeps the middle in one CTA of the solve.
+bool coarse_twist_inv_ok(const Twist& tw, int m) { return tw.H > 0 && tw.mm <= kMidMax && m <= kMidMax; }
+
+static int coarse_ldg(const Twist& tw) { return (tw.mm + 31) / 32 * 32; }
+long long coarse_g_len(const Twist& tw, int m) { return tw.H > 0 ? (long long)m * coarse_ldg(tw) : 0; }
+
 cudaError_t launch_coarse_zinv(int Nc, int m, Buffers& b, cudaStream_t s) {
   const int smem = zinv_smem(m);
   cudaError_t e = raise_smem_limit(k_coarse_zinv, smem);
   if (e != cudaSuccess) return e;
-  k_coarse_zinv<<<(Nc + kZCols - 1) / kZCols, kZT, smem, s>>>(Nc, m, coarse_ring(m), b.f32.Lc, b.f32.Z,
-                                                  coarse_ldz(Nc));
+  const Twist& tw = b.twist;
+  const int N = tw.H > 0 ? tw.Ns : Nc;
+  const long long ldz = coarse_ldz(N);
+  k_coarse_zinv<<<dim3((N + kZCols - 1) / kZCols, tw.H > 0 ? 2 : 1), kZT, smem, s>>>(
+      N, m, tw.H, coarse_ring(m), b.f32.Lc, b.f32.Z, ldz);
   count_launches(1);
+  if (tw.H > 0) {
+    const int mb = m < tw.H ? m : tw.H;
+    k_coarse_g<<<(mb + 3) / 4, kMidMax, 0, s>>>(N, m, tw.H, b.f32.Lc, b.f32.Z, ldz, b.f32.G,
+                                                coarse_ldg(tw));
+    count_launches(1);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_coarse_solve_f32(int Nc, int m, Buffers& b, cudaStream_t s) {
   SingleBuffers& f = b.f32;
-  const long long ldz = coarse_ldz(Nc);
-  const dim3 grid((unsigned)((Nc + kZS - 1) / kZS), (unsigned)((Nc + kZK - 1) / kZK));
-  k_coarse_zlower<<<grid, 256, 0, s>>>(Nc, f.Z, ldz, b.rc, f.zpart);
-  k_coarse_tsum<<<(Nc + 255) / 256, 256, 0, s>>>(Nc, m, f.Lc, f.zpart, ldz, f.tc);
-  k_coarse_zupper<<<(Nc + 7) / 8, 256, 0, s>>>(Nc, f.Z, ldz, f.tc, f.pc);
+  const Twist& tw = b.twist;
+  const int N = tw.H > 0 ? tw.Ns : Nc, bands = tw.H > 0 ? 2 : 1;
+  const long long ldz = coarse_ldz(N);
+  const int chunks = (N + kZK - 1) / kZK;
+  k_coarse_zlower<<<dim3((N + kZS - 1) / kZS, chunks, bands), 256, 0, s>>>(N, Nc, tw.H, f.Z, ldz, b.rc,
+                                                                          f.zpart);
+  if (tw.H > 0) {
+    const int rest = 2 * tw.H - (m < tw.H ? m : tw.H);
+    k_coarse_tsum2<<<1 + (rest + kMidT - 1) / kMidT, kMidT, 0, s>>>(
+        N, m, tw.H, f.Lc, f.G, coarse_ldg(tw), f.zpart, ldz, chunks, f.tc);
+  } else {
+    k_coarse_tsum<<<(Nc + 255) / 256, 256, 0, s>>>(Nc, m, f.Lc, f.zpart, ldz, f.tc);
+  }
+  k_coarse_zupper<<<dim3((N + 7) / 8, bands), 256, 0, s>>>(N, Nc, tw.H, f.Z, ldz, f.tc, f.pc);
   count_launches(3);
   return cudaGetLastError();
 }
