@@ -1615,8 +1615,17 @@ __device__ __forceinline__ double gband_at(const double* B, int m, int r, int c)
   return (r - c <= m && c - r <= m) ? B[(long long)c * (2 * m + 1) + (r - c + m)] : 0.0;
 }
 
-__global__ void __launch_bounds__(256) k_lu_block(int N, int m, int c0, const double* __restrict__ Br,
-                                                  double* B, double* F, int* status) {
+//
+// The block's pivots are a chain (a product, an FMA and a reciprocal each), and
+// the panels' 16 steps run beside it, four threads a row or column as in
+// k_ldlt_block: solved after it by one warp each, whose 136 FP64 instructions
+// hold one unit for 4 us, they made a step of the 1000-node lattice (half-width
+// 111) 16.2 us; now 10.9.
+constexpr int kLuThreads = 384;   // 256 for the block's elements, 64 for the L rows, 64 for the U columns
+
+__global__ void __launch_bounds__(kLuThreads) k_lu_block(int N, int m, int c0,
+                                                         const double* __restrict__ Br, double* B,
+                                                         double* F, int* status) {
   __shared__ double D[kTB][kTB + 1];        // diagonal block: U on and above, work below
   __shared__ double L[kTB][kTB + 1];        // its multipliers l_rq (r > q)
   __shared__ double dinv[kTB];              // 1 / u_qq
@@ -1634,11 +1643,11 @@ __global__ void __launch_bounds__(256) k_lu_block(int N, int m, int c0, const do
   const int r0 = rlo + bi * kTB, cc0 = rlo + bj * kTB;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  {
-    const int r = tid / kTB, q = tid % kTB;
+  if (tid < kTB * kTB) {
+    const int r = tid % kTB, q = tid / kTB;   // (a band column's rows are contiguous)
     D[r][q] = (r < tb && q < tb) ? gband_at(Br, m, c0 + r, c0 + q) : 0.0;
     V[r][q] = (have_tile && r0 + r <= rhi && q < tb) ? gband_at(Br, m, r0 + r, c0 + q) : 0.0;
-    H[q][r] = (have_tile && cc0 + r <= rhi && q < tb) ? gband_at(Br, m, c0 + q, cc0 + r) : 0.0;
+    H[r][q] = (have_tile && cc0 + q <= rhi && r < tb) ? gband_at(Br, m, c0 + r, cc0 + q) : 0.0;
     L[r][q] = 0.0;
   }
   __syncthreads();
@@ -1647,44 +1656,69 @@ __global__ void __launch_bounds__(256) k_lu_block(int N, int m, int c0, const do
     dinv[0] = pivot_rcp_signed(D[0][0], bad);
     if (bad && blockIdx.x == 0) atomicOr(status, kStatSingular);
   }
+  // panels, four threads a row of V (the columns 4 j + pt) or a column of H
+  // (the rows 4 j + pt), in registers
+  const int pk = ((tid - 256) & 63) >> 2, pt = tid & 3, src0 = (tid & 31) & ~3;
+  const bool on_v = tid < 256 + 64;
+  double v[kTB / 4];
+  if (tid >= 256) {
+#pragma unroll
+    for (int j = 0; j < kTB / 4; ++j) v[j] = on_v ? V[pk][4 * j + pt] : H[4 * j + pt][pk];
+  }
   __syncthreads();
-  // --- D = L_D U_D, one element a thread ---
+  // --- D = L_D U_D, one element a thread, pivot by pivot.  Beside it, under
+  // the same barriers: step q of the L panel needs row q of U and 1/u_qq, final
+  // once pivot q - 1 is done, and step q - 1 of the U panel column q - 1 of
+  // L_D, so both run along instead of after it ---
   const int er = tid / kTB, ec = tid % kTB;
-  for (int q = 0; q < tb; ++q) {
-    if (er > q && er < tb) {
-      const double t = D[er][q] * dinv[q];
-      if (ec == q) {
-        L[er][q] = t;
-      } else if (ec > q && ec < tb) {
-        const double v = fma(-t, D[q][ec], D[er][ec]);
-        D[er][ec] = v;
-        if (er == q + 1 && ec == q + 1) {     // the next pivot is final
-          bool bad;
-          dinv[q + 1] = pivot_rcp_signed(v, bad);
-          if (bad && blockIdx.x == 0) atomicOr(status, kStatSingular);
+#pragma unroll
+  for (int q = 0; q < kTB; ++q) {
+    if (q < tb) {                              // uniform across the CTA
+      if (tid < 256) {
+        if (er > q && er < tb && ec >= q && ec < tb) {
+          const double t = D[er][q] * dinv[q];
+          if (ec == q) {
+            L[er][q] = t;
+          } else {
+            const double u = fma(-t, D[q][ec], D[er][ec]);
+            D[er][ec] = u;
+            if (er == q + 1 && ec == q + 1) { // the next pivot is final
+              bool bad;
+              dinv[q + 1] = pivot_rcp_signed(u, bad);
+              if (bad && blockIdx.x == 0) atomicOr(status, kStatSingular);
+            }
+          }
         }
+      } else if (on_v) {
+        double l = 0.0;
+        if (pt == (q & 3)) {
+          l = v[q >> 2] * dinv[q];
+          v[q >> 2] = l;
+        }
+        l = __shfl_sync(0xffffffffu, l, src0 | (q & 3));
+#pragma unroll
+        for (int j = 0; j < kTB / 4; ++j)
+          if (4 * j + 3 > q && 4 * j + pt > q) v[j] = fma(-l, D[q][4 * j + pt], v[j]);
+      } else if (q > 0) {
+        const int p = q - 1;
+        const double u = __shfl_sync(0xffffffffu, v[p >> 2], src0 | (p & 3));
+#pragma unroll
+        for (int j = 0; j < kTB / 4; ++j)
+          if (4 * j + 3 > p && 4 * j + pt > p) v[j] = fma(-L[4 * j + pt][p], u, v[j]);
       }
+      __syncthreads();
     }
-    __syncthreads();
   }
-  // --- panels: row k of V by thread k of warp 0, column k of H by thread k
-  // of warp 1 (two sub-partitions: their FP64 chains run side by side) ---
-  if (tid < kTB) {
-    const int k = tid;
-    for (int q = 0; q < tb; ++q) {
-      double s = V[k][q];
-      for (int j = 0; j < q; ++j) s = fma(-V[k][j], D[j][q], s);
-      V[k][q] = s * dinv[q];
-    }
-  } else if (tid >= 32 && tid < 32 + kTB) {
-    const int k = tid - 32;
-    for (int q = 0; q < tb; ++q) {
-      double s = H[q][k];
-      for (int j = 0; j < q; ++j) s = fma(-L[q][j], H[j][k], s);
-      H[q][k] = s;
+  // (the U panel's last step, p = tb - 1, has no row below it)
+  if (tid >= 256) {
+#pragma unroll
+    for (int j = 0; j < kTB / 4; ++j) {
+      if (on_v) V[pk][4 * j + pt] = v[j];
+      else H[4 * j + pt][pk] = v[j];
     }
   }
   __syncthreads();
+  if (tid >= 256) return;
   if (have_tile) {
     // trailing tile: B[r][c] -= sum_q l_rq u_qc (|r - c| < m inside the window)
     const int a = tid / kTB, bc = tid % kTB;
@@ -2149,7 +2183,7 @@ cudaError_t launch_band_factor(int Nc, int m, int sym, Buffers& b, cudaStream_t 
       const int nb = rhi > c1 ? (rhi - c1 - 1 + kTB) / kTB : 0;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(nb > 0 ? nb * nb : 1);
-      cfg.blockDim = dim3(256);
+      cfg.blockDim = dim3(kLuThreads);
       cfg.dynamicSmemBytes = 0;
       cfg.stream = s;
       cfg.attrs = attr;
