@@ -155,6 +155,7 @@ struct Buffers {
   double* red = nullptr;                                  // reduction partials
   unsigned* tick = nullptr;                               // CTAs that have left theirs; the next entity
   double* scal = nullptr;                                 // reduced scalars (device)
+  double* mail = nullptr;                                 // their copy for the host (host memory)
   int* status = nullptr;                                  // device status word
   SingleBuffers f32;                                      // mixed precision only
 };
@@ -211,7 +212,9 @@ cudaError_t launch_adapt_flags(const Geo& g, const Entity* ents, int count, doub
                                Buffers& b, unsigned char* flag, cudaStream_t s);
 cudaError_t launch_adapt_propagate(const Geo& g, int first, int count, Buffers& b,
                                    cudaStream_t s);
-cudaError_t launch_count_flags(int count, const unsigned char* flag, double* out, cudaStream_t s);
+cudaError_t launch_count_flags(int count, const unsigned char* flag, double* mail, cudaStream_t s);
+// Whether kernels on the device can write ordinary host memory (noalloc.cu).
+bool host_writable(int dev);
 // single: P and the local solves in FP32 (mixed precision), else FP64.
 cudaError_t launch_vertices(const Geo& g, const CGeo& c, Buffers& b, bool single, cudaStream_t s);
 // blocked: panels of pivots with a register-tiled trailing update (large

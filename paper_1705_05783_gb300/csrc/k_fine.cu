@@ -89,7 +89,7 @@ struct AsmIn {
   const unsigned char* fixm;
 };
 struct AsmOut {
-  double *Ad, *Ax, *Ay, *Az, *Cacc, *f, *eps, *Axu, *Ayu, *Azu, *red, *scal;
+  double *Ad, *Ax, *Ay, *Az, *Cacc, *f, *eps, *Axu, *Ayu, *Azu, *red, *scal, *mail;
   unsigned* tick;
 };
 
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kColThreads, 3) k_assemble(
       pi = pzu; ri = rzu; fi = fzu;
     }
   }
-  finish_sum(block_sum(e2), out.red, out.tick, out.scal);
+  if (finish_sum(block_sum(e2), out.red, out.tick, out.scal)) out.mail[0] = out.scal[0];
 }
 
 // Prescribed cells in list order (a repeated cell keeps its last value):
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kColThreads, 4) k_residual(
     const double* __restrict__ Ay, const double* __restrict__ Az, const double* __restrict__ Axu,
     const double* __restrict__ Ayu, const double* __restrict__ Azu, const double* __restrict__ f,
     const double* __restrict__ p, double* r, float* r32, double* red, unsigned* tick, double* scal,
-    LoopCtl ctl) {
+    double* mail, LoopCtl ctl) {
   const double s2 = block_sum(residual_columns(g, w, Ad, Ax, Ay, Az, Axu, Ayu, Azu, f, p, r, r32));
   if (!finish_sum(s2, red, tick, scal)) return;
   if (ctl.mode == LoopCtl::kBegin) {
@@ -294,7 +294,9 @@ __global__ void __launch_bounds__(kColThreads, 4) k_residual(
     const double rn = sqrt(scal[0]), r0 = sqrt(scal[1]);
     const bool more = its < (double)ctl.max_cams && isfinite(rn) && !(rn < ctl.lin_rtol * r0);
     cudaGraphSetConditional(ctl.cond, more ? 1u : 0u);
+    mail[2] = its;
   }
+  mail[0] = scal[0];
 }
 
 // Basis operators A_b (Eqs. 8-11, Reading R10: internal faces only).
@@ -369,7 +371,7 @@ cudaError_t launch_assemble(const Geo& g, const FluidK& fl, double dt, int diric
   const double rhoe = fl.law == 0 ? fl.rho0 * std::exp(fl.c * pe) : fl.rho0 * (1.0 + fl.c * pe);
   const AsmIn in{b.p, b.rho, b.rhon, b.Tx, b.Ty, b.Tz, b.Tbw, b.Tbe, b.src, fixm};
   const AsmOut out{b.Ad, b.Ax, b.Ay, b.Az, b.Cacc, b.f, b.eps, b.Axu, b.Ayu, b.Azu, b.red, b.scal,
-                   b.tick};
+                   b.mail, b.tick};
   auto* kern = fixm ? (full ? k_assemble<true, true> : k_assemble<true, false>)
                     : (full ? k_assemble<false, true> : k_assemble<false, false>);
   const ColWork w = col_work(g);
@@ -396,7 +398,7 @@ cudaError_t launch_residual(const Geo& g, const Buffers& b, cudaStream_t s, cons
   const ColWork w = col_work(g);
   k_residual<<<col_grid(w), kColThreads, 0, s>>>(g, w, b.Ad, b.Ax, b.Ay, b.Az, b.Axu, b.Ayu, b.Azu,
                                                  b.f, b.p, b.r, b.f32.r, b.red, b.tick, b.scal,
-                                                 ctl);
+                                                 b.mail, ctl);
   count_launches(1);
   return cudaGetLastError();
 }

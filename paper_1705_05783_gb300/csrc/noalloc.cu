@@ -114,9 +114,19 @@ __global__ void k_finish_noalloc(int nblocks, const double* scratch, double* tot
   if (threadIdx.x == 0) *total = s;
 }
 
+int fail_na(int code, const std::string& msg) {
+  cams::set_global_error(msg);
+  return code;
+}
+
+}  // namespace
+
+namespace cams {
+
 // Whether kernels on the device can write ordinary host memory.
 bool host_writable(int dev) {
   static std::atomic<int> known[kMaxDevices];   // 0 not asked, 1 no, 2 yes
+  if (dev < 0 || dev >= kMaxDevices) return false;
   int k = known[dev].load(std::memory_order_relaxed);
   if (k == 0) {
     int v = 0;
@@ -127,12 +137,7 @@ bool host_writable(int dev) {
   return k == 2;
 }
 
-int fail_na(int code, const std::string& msg) {
-  cams::set_global_error(msg);
-  return code;
-}
-
-}  // namespace
+}  // namespace cams
 
 extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* diag,
                                           const double* ax, const double* ay, const double* az,
@@ -175,7 +180,7 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
   // tables), the total goes straight to it and the stream's end makes it
   // visible; a copy of the eight bytes takes 5 to 10 us more.
   double s2 = 0.0;
-  const bool direct = norm_out && host_writable(dev);
+  const bool direct = norm_out && cams::host_writable(dev);
   double* total = direct ? &s2 : scratch + kMaxBlocks;
   cams::ColWork w = cams::col_work(g, kSmallThreads);
   if (w.pieces <= (unsigned)kSmallPieces) {
