@@ -1862,9 +1862,12 @@ __global__ void __launch_bounds__(256) k_restrict_fe_local(Geo g, CGeo c, const 
 }
 
 // MSFE restriction, part 2: coarse node J sums its (up to 8) dual blocks.
+// It also clears the abort flag of the coarse solve that follows (a memset of
+// its own was a node of every iteration's graph).
 __global__ void k_restrict_fe_gather(CGeo c, const double* __restrict__ part, const int* __restrict__ perm,
-                                     double* rc) {
+                                     double* rc, int* abort_flag) {
   const int J = blockIdx.x * blockDim.x + threadIdx.x;
+  if (J == 0) *abort_flag = 0;
   if (J >= c.Nc) return;
   const int Jc[3] = {J % c.nc[0], (J / c.nc[0]) % c.nc[1], J / (c.nc[0] * c.nc[1])};
   const int ndx = c.nc[0] + 1, ndy = c.nc[1] + 1;
@@ -2225,7 +2228,8 @@ cudaError_t launch_restrict(const Geo& g, const CGeo& c, int kind, const double*
     else if (single) k_restrict_fe_local<float, double><<<nd, block_threads(c), 0, s>>>(g, c, b.f32.P, r, b.loc);
     else k_restrict_fe_local<double, double><<<nd, block_threads(c), 0, s>>>(g, c, b.P, r, b.loc);
     count_launches(1);
-    k_restrict_fe_gather<<<(c.Nc + 127) / 128, 128, 0, s>>>(c, b.loc, b.perm, b.rc); count_launches(1);
+    k_restrict_fe_gather<<<(c.Nc + 127) / 128, 128, 0, s>>>(c, b.loc, b.perm, b.rc, b.cabort);
+    count_launches(1);
   } else {
     k_restrict_fv<<<c.Nc, block_threads(c), 0, s>>>(g, c, r, b.perm, b.rc); count_launches(1);
   }
@@ -2286,8 +2290,8 @@ bool coarse_cluster_ok(int Nc, int max_smem) {
 cudaError_t launch_band_solve(int Nc, int m, int sym, bool cluster, bool single, Buffers& b,
                               cudaStream_t s) {
   if (sym && cluster) {
-    cudaError_t e = cudaMemsetAsync(b.cabort, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
+    // (the restriction that formed b.rc cleared b.cabort)
+    cudaError_t e = cudaSuccess;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kCC);
     cfg.blockDim = dim3(256);
