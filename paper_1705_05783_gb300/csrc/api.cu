@@ -810,7 +810,7 @@ int cams_step_direct(cams_handle* h) {
   if (h->coarse_inv)
     LAUNCH(CAMS_PROF_COARSE_SOLVE, launch_coarse_solve_f32(h->c.Nc, h->mc, b, h->stream));
   else
-    LAUNCH(CAMS_PROF_COARSE_SOLVE, launch_band_solve(h->c.Nc, h->mc, !fv && !h->opt.jacobian,
+    LAUNCH(CAMS_PROF_COARSE_SOLVE, launch_band_solve(h->g, h->c.Nc, h->mc, !fv && !h->opt.jacobian,
                                                      h->coarse_cluster, s, b, h->stream));
   LAUNCH(CAMS_PROF_PROLONG, launch_prolong_add(h->g, h->c, s, b, h->stream));
   for (int k = 0; k < h->opt.n_post; ++k) {
@@ -1374,7 +1374,7 @@ int closing_msfv(cams_handle* h) {
   }
   LAUNCH(CAMS_PROF_RESIDUAL, launch_residual(h->g, b, h->stream));
   LAUNCH(CAMS_PROF_RESTRICT, launch_restrict(h->g, h->c, 1, b.r, h->single, b, h->stream));
-  LAUNCH(CAMS_PROF_COARSE_SOLVE, launch_band_solve(h->c.Nc, h->mc, 0, false, false, b, h->stream));
+  LAUNCH(CAMS_PROF_COARSE_SOLVE, launch_band_solve(h->g, h->c.Nc, h->mc, 0, false, false, b, h->stream));
   LAUNCH(CAMS_PROF_PROLONG, launch_prolong_to_p(h->g, h->c, h->single, b, h->stream));
   return check_status(h);
 }

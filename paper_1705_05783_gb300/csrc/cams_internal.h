@@ -262,8 +262,8 @@ cudaError_t launch_restrict(const Geo& g, const CGeo& c, int kind, const double*
 // the coarse solution into b.pc; with single into b.f32.pc for the FP32
 // prolongation (the symmetric cluster solve then substitutes in FP32 with
 // the FP32 copy of the factor)
-cudaError_t launch_band_solve(int Nc, int m, int sym, bool cluster, bool single, Buffers& b,
-                              cudaStream_t s);
+cudaError_t launch_band_solve(const Geo& g, int Nc, int m, int sym, bool cluster, bool single,
+                              Buffers& b, cudaStream_t s);
 long long coarse_blocks_len(int Nc);
 bool coarse_cluster_ok(int Nc, int max_smem);
 Twist coarse_twist(int Nc, int m);

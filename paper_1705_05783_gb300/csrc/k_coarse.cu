@@ -14,6 +14,7 @@
 // block tree, and every sum over blocks runs in a fixed block order, so the
 // MSFE matrix is bitwise symmetric.
 #include "cams_internal.h"
+#include "launch.h"
 #include "rcp64.h"
 
 namespace cams {
@@ -1282,6 +1283,7 @@ __global__ void __launch_bounds__(256, 1) k_coarse_solve_cluster(
   const int tid = threadIdx.x, r = tid >> 3, h = tid & 7;
   const int W = (m + kCB - 1) / kCB;           // blocks of the band left of a diagonal block
   for (int i = tid; i < 2 * Np; i += blockDim.x) sm[i] = CWord<T>::value(CWord<T>::kNR);
+  pdl_enter();
   cl_sync();
   bool ok = true;
   // ---- forward: L y = b ----
@@ -1425,6 +1427,7 @@ __global__ void __launch_bounds__(256, 1) k_coarse_solve_twisted(
   const int W = (m + kCB - 1) / kCB;
   for (int i = tid; i < 4 * Np; i += blockDim.x)
     sm[i] = i >= 3 * Np + Ns ? T(0) : CWord<T>::value(CWord<T>::kNR);
+  pdl_enter();
   cl_sync();
   bool ok = true;
   // ---- forward ----
@@ -1829,6 +1832,7 @@ template <class TP, class TR>
 __global__ void __launch_bounds__(256) k_restrict_fe_local(Geo g, CGeo c, const TP* __restrict__ P,
                                                            const TR* __restrict__ r, double* part) {
   __shared__ double sh[8 * 8];
+  pdl_enter();
   const int ndx = c.nc[0] + 1, ndy = c.nc[1] + 1;
   const int D = blockIdx.x;
   const int j[3] = {D % ndx, (D / ndx) % ndy, D / (ndx * ndy)};
@@ -1866,6 +1870,7 @@ __global__ void __launch_bounds__(256) k_restrict_fe_local(Geo g, CGeo c, const 
 // its own was a node of every iteration's graph).
 __global__ void k_restrict_fe_gather(CGeo c, const double* __restrict__ part, const int* __restrict__ perm,
                                      double* rc, int* abort_flag) {
+  pdl_enter();
   const int J = blockIdx.x * blockDim.x + threadIdx.x;
   if (J == 0) *abort_flag = 0;
   if (J >= c.Nc) return;
@@ -1924,6 +1929,7 @@ template <class TP, class TC, class TO, bool kSet>
 __global__ void k_prolong(Geo g, CGeo c, const TP* __restrict__ P, const TC* __restrict__ pc,
                           const int* __restrict__ perm, const int* __restrict__ jxt, TO* p) {
   extern __shared__ __align__(16) unsigned char prolong_smem[];
+  pdl_enter();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int ncx = c.nc[0];
   TC* cv = reinterpret_cast<TC*>(prolong_smem) + (size_t)warp * 4 * ncx;
@@ -2226,10 +2232,14 @@ cudaError_t launch_restrict(const Geo& g, const CGeo& c, int kind, const double*
     // mixed precision: the FP32 copy of the handle's residual (written with it)
     if (single && r == b.r) k_restrict_fe_local<float, float><<<nd, block_threads(c), 0, s>>>(g, c, b.f32.P, b.f32.r, b.loc);
     else if (single) k_restrict_fe_local<float, double><<<nd, block_threads(c), 0, s>>>(g, c, b.f32.P, r, b.loc);
-    else k_restrict_fe_local<double, double><<<nd, block_threads(c), 0, s>>>(g, c, b.P, r, b.loc);
-    count_launches(1);
-    k_restrict_fe_gather<<<(c.Nc + 127) / 128, 128, 0, s>>>(c, b.loc, b.perm, b.rc, b.cabort);
-    count_launches(1);
+    else {
+      const cudaError_t e = launch_after(pdl_grid(g), k_restrict_fe_local<double, double>, dim3(nd),
+                                         block_threads(c), 0, s, g, c, b.P, r, b.loc);
+      if (e != cudaSuccess) return e;
+    }
+    count_launches(2);
+    return launch_after(pdl_grid(g), k_restrict_fe_gather, dim3((c.Nc + 127) / 128), 128, 0, s, c, b.loc,
+                        b.perm, b.rc, b.cabort);
   } else {
     k_restrict_fv<<<c.Nc, block_threads(c), 0, s>>>(g, c, r, b.perm, b.rc); count_launches(1);
   }
@@ -2287,8 +2297,8 @@ bool coarse_cluster_ok(int Nc, int max_smem) {
   return n > 0;
 }
 
-cudaError_t launch_band_solve(int Nc, int m, int sym, bool cluster, bool single, Buffers& b,
-                              cudaStream_t s) {
+cudaError_t launch_band_solve(const Geo& g, int Nc, int m, int sym, bool cluster, bool single,
+                              Buffers& b, cudaStream_t s) {
   if (sym && cluster) {
     // (the restriction that formed b.rc cleared b.cabort)
     cudaError_t e = cudaSuccess;
@@ -2297,13 +2307,14 @@ cudaError_t launch_band_solve(int Nc, int m, int sym, bool cluster, bool single,
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = (size_t)coarse_cluster_smem(Nc, single ? 4 : 8);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kCC;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl_grid(g) ? 2 : 1;
     const Twist& tw = b.twist;
     if (tw.H > 0) {
       const SingleBuffers& f = b.f32;
@@ -2375,9 +2386,9 @@ static cudaError_t prolong(const Geo& g, const CGeo& c, const TP* P, const TC* p
     if (e != cudaSuccess) return e;
   }
   const int blocks = (int)(((long long)g.ny * g.nz + w - 1) / w);   // one warp per x-row
-  k_prolong<TP, TC, TO, kSet><<<blocks, 32 * w, smem, s>>>(g, c, P, pc, b.perm, b.jxt, p);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_after(pdl_grid(g), k_prolong<TP, TC, TO, kSet>, dim3(blocks), 32 * w, smem, s, g, c, P, pc,
+                      b.perm, b.jxt, p);
 }
 
 cudaError_t launch_prolong_add(const Geo& g, const CGeo& c, bool single, Buffers& b,

@@ -7,6 +7,7 @@
 // of a warp is a coalesced 256-byte run; the neighbour reads of the 7-point
 // stencil hit L1/L2.  FP64 throughout.
 #include "cams_internal.h"
+#include "launch.h"
 #include "rcp64.h"
 #include "stencil.h"
 
@@ -283,6 +284,7 @@ __global__ void __launch_bounds__(kColThreads, 4) k_residual(
     const double* __restrict__ Ayu, const double* __restrict__ Azu, const double* __restrict__ f,
     const double* __restrict__ p, double* r, float* r32, double* red, unsigned* tick, double* scal,
     double* mail, LoopCtl ctl) {
+  pdl_enter();
   const double s2 = block_sum(residual_columns(g, w, Ad, Ax, Ay, Az, Axu, Ayu, Azu, f, p, r, r32));
   if (!finish_sum(s2, red, tick, scal)) return;
   if (ctl.mode == LoopCtl::kBegin) {
@@ -396,11 +398,9 @@ cudaError_t launch_fix_cells(int n, const int* cell, const double* val, unsigned
 
 cudaError_t launch_residual(const Geo& g, const Buffers& b, cudaStream_t s, const LoopCtl& ctl) {
   const ColWork w = col_work(g);
-  k_residual<<<col_grid(w), kColThreads, 0, s>>>(g, w, b.Ad, b.Ax, b.Ay, b.Az, b.Axu, b.Ayu, b.Azu,
-                                                 b.f, b.p, b.r, b.f32.r, b.red, b.tick, b.scal,
-                                                 b.mail, ctl);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_after(pdl_grid(g), k_residual, dim3(col_grid(w)), kColThreads, 0, s, g, w, b.Ad, b.Ax, b.Ay,
+                      b.Az, b.Axu, b.Ayu, b.Azu, b.f, b.p, b.r, b.f32.r, b.red, b.tick, b.scal, b.mail, ctl);
 }
 
 cudaError_t launch_basis_operator(const Geo& g, const FluidK& fl, int kind, double dt,

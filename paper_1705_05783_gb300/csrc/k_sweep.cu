@@ -58,6 +58,7 @@
 //  The backward sweep runs the same schedule on the mirrored grid: its steps
 //  read the same records in reverse order.
 #include "cams_internal.h"
+#include "launch.h"
 
 namespace cams {
 
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(256) k_resid_scaled(Geo g, Shape s, const T* _
   constexpr int G = L::G, kRows = 32, kC = kXC<T>;
   __shared__ alignas(16) T blk[kRows][kRow<T>];
   const int tile = blockIdx.x, x0 = blockIdx.y * kC;
+  pdl_enter();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 3) ctrl[threadIdx.x] = 0;
   const int Y = tile % s.nty, Z = tile / s.nty;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(256) k_apply_z(Geo g, Shape s, const T* __rest
   constexpr int G = L::G, kRows = 32, kC = kXC<T>;
   __shared__ alignas(16) T blk[kRows][kRow<T>];
   const int tile = blockIdx.x, x0 = blockIdx.y * kC;
+  pdl_enter();
   const int Y = tile % s.nty, Z = tile / s.nty;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ty = lane % L::TY, tz = lane / L::TY, X0 = x0 / G;
@@ -855,6 +858,7 @@ __global__ void __launch_bounds__(Plan<T, kFlat>::kThreads)
   const unsigned base = (unsigned)__cvta_generic_to_shared(smem_raw), words = base + Pl::kCtrl;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned rank = cluster_rank();
+  pdl_enter();
   // (a ring slot is reset when its chunk is taken, so the rings are unset
   // again after every tile)
   for (int k = threadIdx.x; k < Pl::kRingsB / Pl::kV; k += blockDim.x)
@@ -950,7 +954,7 @@ IluSet<float> set_of(Buffers& b, float*) {
 
 // cta: blocks of kBlock tiles per cluster, else one tile per CTA on its own.
 template <class T, bool kBackward, bool kFlat>
-cudaError_t run_sweep(const Shape& sh, const IluSet<T>& v, bool cta, int* ctrl, int* status,
+cudaError_t run_sweep(const Geo& g, const Shape& sh, const IluSet<T>& v, bool cta, int* ctrl, int* status,
                       cudaStream_t s) {
   using Pl = Plan<T, kFlat>;
   // 8 CTAs a cluster (the portable limit).  Measured at 200 x 200 x 100, FP32 /
@@ -962,12 +966,13 @@ cudaError_t run_sweep(const Shape& sh, const IluSet<T>& v, bool cta, int* ctrl, 
   c.blockDim = dim3(Pl::kThreads);
   c.dynamicSmemBytes = Pl::kBytes;
   c.stream = s;
-  cudaLaunchAttribute a[1];
+  cudaLaunchAttribute a[2];
   a[0].id = cudaLaunchAttributeClusterDimension;
   a[0].val.clusterDim.x = (unsigned)(nby * nbz);
   a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+  a[1] = pdl_attribute();
   c.attrs = a;
-  c.numAttrs = 1;
+  c.numAttrs = pdl_grid(g) ? 2 : 1;
   return cudaLaunchKernelEx(&c, k_sweep<T, kBackward, kFlat>, sh, (const T*)(kBackward ? v.up : v.lo),
                             kBackward ? v.z : v.up, kBackward ? v.up : v.z, ctrl, status, nby, nbz);
 }
@@ -987,8 +992,8 @@ cudaError_t sweep_impl(const Geo& g, Buffers& b, bool backward, bool pipelined, 
     return cudaGetLastError();
   }
   count_launches(1);
-  return backward ? run_sweep<T, true, kFlat>(sh, v, cta, b.ctrl, b.status, s)
-                  : run_sweep<T, false, kFlat>(sh, v, cta, b.ctrl, b.status, s);
+  return backward ? run_sweep<T, true, kFlat>(g, sh, v, cta, b.ctrl, b.status, s)
+                  : run_sweep<T, false, kFlat>(g, sh, v, cta, b.ctrl, b.status, s);
 }
 
 template <class T, bool kFlat>
@@ -996,14 +1001,10 @@ cudaError_t resid_impl(const Geo& g, Buffers& b, cudaStream_t s) {
   const Shape sh = shape_of<T, kFlat>(g);
   const IluSet<T> v = set_of(b, (T*)nullptr);
   const dim3 grid(sh.nty * sh.ntz, (g.nx + kXC<T> - 1) / kXC<T>);
-  if (v.Axu != v.Ax)
-    k_resid_scaled<T, true, kFlat><<<grid, 256, 0, s>>>(g, sh, v.Ad, v.Ax, v.Ay, v.Az, v.Axu, v.Ayu,
-                                                       v.Azu, v.b, v.x, v.dinv, v.lo, b.ctrl);
-  else
-    k_resid_scaled<T, false, kFlat><<<grid, 256, 0, s>>>(g, sh, v.Ad, v.Ax, v.Ay, v.Az, v.Axu, v.Ayu,
-                                                        v.Azu, v.b, v.x, v.dinv, v.lo, b.ctrl);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_after(pdl_grid(g), v.Axu != v.Ax ? k_resid_scaled<T, true, kFlat> : k_resid_scaled<T, false, kFlat>,
+                      grid, 256, 0, s, g, sh, v.Ad, v.Ax, v.Ay, v.Az, v.Axu, v.Ayu, v.Azu, v.b, v.x,
+                      v.dinv, v.lo, b.ctrl);
 }
 
 template <class T, bool kFlat>
@@ -1011,9 +1012,8 @@ cudaError_t apply_impl(const Geo& g, Buffers& b, cudaStream_t s) {
   const Shape sh = shape_of<T, kFlat>(g);
   const IluSet<T> v = set_of(b, (T*)nullptr);
   const dim3 grid(sh.nty * sh.ntz, (g.nx + kXC<T> - 1) / kXC<T>);
-  k_apply_z<T, kFlat><<<grid, 256, 0, s>>>(g, sh, v.z, v.x);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_after(pdl_grid(g), k_apply_z<T, kFlat>, grid, 256, 0, s, g, sh, v.z, v.x);
 }
 
 template <class T, bool kFlat>

@@ -1,0 +1,45 @@
+// Launches that may begin while the kernel before them drains (programmatic
+// dependent launch): the CTAs are placed early and wait in pdl_enter until
+// that kernel has completed and its writes are visible.
+#pragma once
+
+#include "cams_internal.h"
+
+namespace cams {
+
+// Grids whose iteration is a chain of kernels of a few microseconds, where the
+// gaps between them count.  Larger ones would only hold SMs while they wait, which other
+// members of an ensemble could use.
+inline bool pdl_grid(const Geo& g) { return g.N <= 20000; }
+
+#ifdef __CUDACC__
+// At the top of a kernel that is launched so, before any access to memory
+// (both are no-ops in an ordinary launch).
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+inline cudaLaunchAttribute pdl_attribute() {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+
+template <class... P, class... A>
+cudaError_t launch_after(bool pdl, void (*kern)(P...), dim3 grid, int threads, int smem, cudaStream_t s,
+                         A&&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = (size_t)smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  c.attrs = at;
+  c.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+#endif
+
+}  // namespace cams
