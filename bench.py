@@ -69,7 +69,9 @@ T_STEP_US = {0: 0.78 / 4, 1: 0.30 / 4}
 SWEEP_CLASSES = ("ilu_fwd", "ilu_bwd")
 
 # DRAM bytes per launch measured by ncu (dram__bytes_read.sum + write.sum) for
-# a kernel class on a workload, for the kernels as they stand; see profiles/.
+# a kernel class on a workload; see profiles/.  (Measured with the sweeps of one
+# tile a warp; the cluster sweeps read and write the same operands:
+# profiles/launch_list_3d-200x200x100-mixed-clusters.md.)
 MEASURED_TRAFFIC = {
     # profiles/launch_list_3d-200x200x100-mixed.md (the kernels as of the FP32 residual copy)
     ("3d-200x200x100-mixed", "ilu_fwd"): 73.9e6,

@@ -8,8 +8,10 @@
 namespace cams {
 
 // Grids whose iteration is a chain of kernels of a few microseconds, where the
-// gaps between them count.  Larger ones would only hold SMs while they wait, which other
-// members of an ensemble could use.
+// gaps between them count (five steps at 40x40: 21.4 -> 20.7 ms).  On larger
+// ones the waiting CTAs hold SMs that the kernel before them, or other members
+// of an ensemble, could use: with every grid launched so a 64^3 step took 18.2
+// ms instead of 17.3 and 16 members 110 instead of 91.
 inline bool pdl_grid(const Geo& g) { return g.N <= 20000; }
 
 #ifdef __CUDACC__
