@@ -325,9 +325,9 @@ cudaError_t launch_energy(int B, int S, int C, int cx, const float* p, const flo
 int mse_partial_blocks();
 // Tensor-core (tcgen05, BF16 operands, FP32 accumulation) path of the
 // network (k_net_tc.cu).  Activations between layers are BF16 "chunked and
-// padded" (a zero border around the patch, channels in chunks of 8); a
-// buffer of net_tc_act_elems(B, S, C) BF16 values must start zeroed (only
-// rows inside the output-tile range are ever written).
+// padded" (a zero border around the patch, channels in chunks of 8); a layer
+// writes every row of its buffer of net_tc_act_elems(B, S, C) BF16 values, the
+// border too.
 long long net_tc_act_elems(int B, int S, int C);
 bool net_tc_fits(int S, int max_smem);
 // FP32 [B][C][S^3] -> BF16 chunked-padded
