@@ -489,8 +489,15 @@ __device__ __forceinline__ unsigned map_rank(unsigned p, unsigned rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(q) : "r"(p), "r"(rank));
   return q;
 }
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ void store_cluster(unsigned p, int v) {
   asm volatile("st.relaxed.cluster.shared::cluster.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
@@ -858,11 +865,14 @@ __global__ void __launch_bounds__(Plan<T, kFlat>::kThreads)
   const unsigned base = (unsigned)__cvta_generic_to_shared(smem_raw), words = base + Pl::kCtrl;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned rank = cluster_rank();
+  cluster_arrive();
   pdl_enter();
   // (a ring slot is reset when its chunk is taken, so the rings are unset
   // again after every tile)
   for (int k = threadIdx.x; k < Pl::kRingsB / Pl::kV; k += blockDim.x)
     Ch::store_shared(base + Pl::kRings + (unsigned)k * Pl::kV, Ch::splat(Ch::unset_value()));
+  // no CTA's shared memory is written from another one before all have started
+  cluster_wait();
   const int ncy = (sh.nty + nby - 1) / nby, ncz = (sh.ntz + nbz - 1) / nbz, nblocks = ncy * ncz;
   Place pc{0, 0, (int)rank % nby, (int)rank / nby, nby, nbz};
   for (unsigned turn = 0;; turn ^= 1u) {
