@@ -22,6 +22,7 @@
 #include <cmath>
 #include <mutex>
 #include <string>
+#include <utility>
 
 #include <cooperative_groups.h>
 
@@ -90,13 +91,12 @@ __global__ void __launch_bounds__(kSmallThreads) k_residual_small(
     const double* __restrict__ Ay, const double* __restrict__ Az, const double* __restrict__ f,
     const double* __restrict__ p, double* r, double* total) {
   __shared__ double part[kSmallCtas];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  // (CTA 0's shared memory is written once it is known to have started)
+  auto started = cl.barrier_arrive();
   const double s2 = cams::block_sum(
       cams::residual_columns(g, w, Ad, Ax, Ay, Az, Ax, Ay, Az, f, p, r, nullptr));
-  if (gridDim.x == 1) {
-    if (threadIdx.x == 0) *total = s2;
-    return;
-  }
-  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.barrier_wait(std::move(started));
   if (threadIdx.x == 0) cl.map_shared_rank(part, 0)[blockIdx.x] = s2;
   cl.sync();
   if (blockIdx.x == 0 && threadIdx.x == 0) {

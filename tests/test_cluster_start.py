@@ -14,7 +14,7 @@ BARRIER = re.compile(r"\bcluster_sync\(\)|\bcluster_wait\(\)|\bcl_sync\(\)|\bcl\
 
 
 def _kernels():
-    for path in sorted(glob.glob(os.path.join(CSRC, "k_*.cu"))):
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
         src = re.sub(r"//[^\n]*", "", open(path).read())
         for m in re.finditer(r"__global__", src):
             depth, start = 0, None
@@ -39,7 +39,8 @@ REACH = [(name, body) for name, body in _kernels() if REMOTE.search(body)]
 
 
 def test_the_cluster_kernels_are_found():
-    assert {n.split(":")[1] for n, _ in REACH} >= {"k_sweep", "k_coarse_solve_cluster", "k_coarse_solve_twisted"}
+    assert {n.split(":")[1] for n, _ in REACH} >= {"k_sweep", "k_residual_small", "k_coarse_solve_cluster",
+                                                   "k_coarse_solve_twisted"}
 
 
 @pytest.mark.parametrize("name, body", REACH, ids=[n for n, _ in REACH])
