@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 
 #include "cams_internal.h"
+#include "launch.h"
 #include "stencil.h"
 
 namespace {
@@ -178,10 +179,13 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // Where the GPU can write this thread's stack (it shares the host's page
   // tables), the total goes straight to it and the stream's end makes it
-  // visible; a copy of the eight bytes takes 5 to 10 us more.
+  // visible; a copy of the eight bytes takes 5 to 10 us more.  So nothing below
+  // returns before the stream is done, and a launch is judged by its own code: an
+  // earlier call's error, still pending in the runtime, is not this one's.
   double s2 = 0.0;
   const bool direct = norm_out && cams::host_writable(dev);
   double* total = direct ? &s2 : scratch + kMaxBlocks;
+  const char* what = "launch: ";
   cams::ColWork w = cams::col_work(g, kSmallThreads);
   if (w.pieces <= (unsigned)kSmallPieces) {
     int ctas = 1;
@@ -196,24 +200,27 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = ctas > 1 ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, k_residual_small, g, w, diag, ax, ay, az, f, p, r, total);
+    e = cudaLaunchKernelEx(&cfg, k_residual_small, g, w, diag, ax, ay, az, f, p, r, total);
     cams::count_launches(1);
   } else {
     w = cams::col_work(g);
     const int nblocks = cams::col_grid(w);
-    k_residual_noalloc<<<nblocks, cams::kColThreads, 0, s>>>(g, w, diag, ax, ay, az, f, p, r,
-                                                              scratch);
-    k_finish_noalloc<<<1, 1024, 0, s>>>(nblocks, scratch, total);
+    e = cams::launch_after(false, k_residual_noalloc, dim3(nblocks), cams::kColThreads, 0, s, g, w, diag,
+                           ax, ay, az, f, p, r, scratch);
+    if (e == cudaSuccess)
+      e = cams::launch_after(false, k_finish_noalloc, dim3(1), 1024, 0, s, nblocks, scratch, total);
     cams::count_launches(2);
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return fail_na(CAMS_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
-  if (norm_out && !direct) {
+  if (e == cudaSuccess && norm_out && !direct) {
+    what = "read-back: ";
     e = cudaMemcpyAsync(&s2, total, sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return fail_na(CAMS_ECUDA, std::string("read-back: ") + cudaGetErrorString(e));
   }
-  e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return fail_na(CAMS_ECUDA, std::string("synchronize: ") + cudaGetErrorString(e));
+  const cudaError_t done = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) {
+    what = "synchronize: ";
+    e = done;
+  }
+  if (e != cudaSuccess) return fail_na(CAMS_ECUDA, std::string(what) + cudaGetErrorString(e));
   if (norm_out) *norm_out = std::sqrt(*static_cast<volatile double*>(&s2));
   return CAMS_OK;
 }

@@ -88,3 +88,24 @@ def test_assembly_on_runs_of_planes(cams, case, jacobian):
         assert abs(eps - want) <= 1e-11 * want
     finally:
         cams.cams_destroy(h)
+
+
+@pytest.mark.parametrize("n", [(256, 256, 256), (40, 40, 1)])
+def test_noalloc_residual_after_another_calls_error(cams, n):
+    """An error left pending by an earlier call (a convolution that no CTA's
+    shared memory holds: refused by the host, nothing launched) is not the
+    residual's: the call succeeds, and its kernels are done when it returns."""
+    import torch
+    N = int(np.prod(n))
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    args = [torch.rand(N, generator=gen, device="cuda", dtype=torch.float64) for _ in range(6)]
+    s = torch.cuda.current_stream()
+    want = cams.cams_residual_norm_noalloc(*n, *args, None, s.cuda_stream)
+    assert want[0] == cams.CAMS_OK
+    t = torch.zeros(16, device="cuda")
+    with pytest.raises(cams.CamsError):
+        cams.cams_net_conv_forward(1, 40, 5000, 1, t, t, t, 0, t)
+    torch.cuda.synchronize()
+    got = cams.cams_residual_norm_noalloc(*n, *args, None, s.cuda_stream)
+    assert s.query()
+    assert got == want
