@@ -107,12 +107,11 @@ __global__ void __launch_bounds__(kColThreads, 3) k_assemble(
   const double ccst = vphidt * (fl.law == 0 ? fl.c : dlin);
   double e2 = 0.0;
   for (unsigned w0 = blockIdx.x; w0 < w.pieces; w0 += gridDim.x) {
-    const unsigned seg = w0 / w.tiles;
-    const long long j = (long long)(w0 - seg * w.tiles) * kColThreads + threadIdx.x;
-    if (j >= g.sz) continue;
-    const unsigned y = (unsigned)j / (unsigned)g.nx, x = (unsigned)j - y * (unsigned)g.nx;
+    unsigned j;
+    int z0, z1;
+    if (!col_of(g, w, w0, j, z0, z1)) continue;
+    const unsigned y = j / (unsigned)g.nx, x = j - y * (unsigned)g.nx;
     const bool xl = x > 0, xu = x + 1 < (unsigned)g.nx, yl = y > 0, yu = y + 1 < (unsigned)g.ny;
-    const int z0 = (int)seg * w.planes, z1 = min(z0 + w.planes, g.nz);
     long long i = j + g.sz * z0;
     double pi = p[i], ri = rho[i];
     bool fi = kFix && in.fixm[i];

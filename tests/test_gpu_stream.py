@@ -109,3 +109,53 @@ def test_noalloc_residual_after_another_calls_error(cams, n):
     got = cams.cams_residual_norm_noalloc(*n, *args, None, s.cuda_stream)
     assert s.query()
     assert got == want
+
+
+# planes of fewer columns than a CTA has threads: one column, fewer than a warp,
+# a CTA and a bit more, with runs of one plane and of several
+@pytest.mark.parametrize("n", [(1, 1, 1025), (1, 1, 1000003), (2, 3, 4001), (4, 4, 65537), (5, 7, 30011), (17, 17, 4099),
+                               (33, 33, 67)])
+def test_noalloc_residual_of_thin_grids(cams, n):
+    import torch
+    nx, ny, nz = n
+    N, eps = nx * ny * nz, np.finfo(float).eps
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    d, ax, ay, az, f, p = (torch.rand(N, generator=gen, device="cuda", dtype=torch.float64) - 0.3 for _ in range(6))
+    i = torch.arange(N, device="cuda")
+    want, mag = f - d * p, f.abs() + (d * p).abs()
+    for a, st, c in ((ax, 1, i % nx), (ay, nx, i // nx % ny), (az, nx * ny, i // (nx * ny))):
+        up = i[c > 0]                                  # the face between up - st and up
+        t = a[up] * p[up - st]
+        want[up] -= t
+        mag[up] += t.abs()
+        t = a[up] * p[up]
+        want[up - st] -= t
+        mag[up - st] += t.abs()
+        a[c == 0] = float("nan")                       # outside the grid: never used
+    r = torch.full((N,), float("nan"), device="cuda", dtype=torch.float64)
+    code, norm = cams.cams_residual_norm_noalloc(nx, ny, nz, d, ax, ay, az, f, p, r,
+                                                 torch.cuda.current_stream().cuda_stream)
+    assert code == cams.CAMS_OK
+    assert bool(((r - want).abs() <= 32 * eps * mag).all())
+    assert abs(norm - r.norm().item()) <= 1e-12 * norm
+
+
+def test_a_thin_grid_costs_as_much_as_a_long_one(cams):
+    """A column of 10^6 cells along z takes no more than five times what the
+    same cells along x do (30 times with a CTA for every plane of one cell)."""
+    import torch
+    N = 1000000
+    args = [torch.ones(N, device="cuda", dtype=torch.float64) for _ in range(6)]
+    s = torch.cuda.current_stream()
+
+    def best(n):
+        times = []
+        for _ in range(8):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record(s)
+            assert cams.cams_residual_norm_noalloc(*n, *args, None, s.cuda_stream)[0] == cams.CAMS_OK
+            b.record(s)
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+    assert best((1, 1, N)) <= 5 * best((N, 1, 1))
