@@ -270,9 +270,10 @@ __global__ void __launch_bounds__(256) k_resid_scaled(Geo g, Shape s, const T* _
   using V = typename Ch::V;
   constexpr int G = L::G, kRows = 32, kC = kXC<T>;
   __shared__ alignas(16) T blk[kRows][kRow<T>];
-  const int tile = blockIdx.x, x0 = blockIdx.y * kC;
+  const int piece = (int)blockIdx.x / (s.nty * s.ntz), tile = (int)blockIdx.x - piece * (s.nty * s.ntz);
+  const int x0 = piece * kC;
   pdl_enter();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 3) ctrl[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 3) ctrl[threadIdx.x] = 0;
   const int Y = tile % s.nty, Z = tile / s.nty;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // (unrolled, with predicates instead of early exits, so that a thread's
@@ -343,7 +344,8 @@ __global__ void __launch_bounds__(256) k_apply_z(Geo g, Shape s, const T* __rest
   using V = typename Ch::V;
   constexpr int G = L::G, kRows = 32, kC = kXC<T>;
   __shared__ alignas(16) T blk[kRows][kRow<T>];
-  const int tile = blockIdx.x, x0 = blockIdx.y * kC;
+  const int piece = (int)blockIdx.x / (s.nty * s.ntz), tile = (int)blockIdx.x - piece * (s.nty * s.ntz);
+  const int x0 = piece * kC;
   pdl_enter();
   const int Y = tile % s.nty, Z = tile / s.nty;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1006,11 +1008,18 @@ cudaError_t sweep_impl(const Geo& g, Buffers& b, bool backward, bool pipelined, 
                   : run_sweep<T, false, kFlat>(g, sh, v, cta, b.ctrl, b.status, s);
 }
 
+// The CTAs of a layout conversion, the tiles of one piece of x after another (in
+// one dimension of the grid: a second one would end at 65535 pieces).
+template <class T>
+dim3 layout_grid(const Geo& g, const Shape& sh) {
+  return dim3((unsigned)(sh.nty * sh.ntz) * (unsigned)((g.nx + kXC<T> - 1) / kXC<T>));
+}
+
 template <class T, bool kFlat>
 cudaError_t resid_impl(const Geo& g, Buffers& b, cudaStream_t s) {
   const Shape sh = shape_of<T, kFlat>(g);
   const IluSet<T> v = set_of(b, (T*)nullptr);
-  const dim3 grid(sh.nty * sh.ntz, (g.nx + kXC<T> - 1) / kXC<T>);
+  const dim3 grid = layout_grid<T>(g, sh);
   count_launches(1);
   return launch_after(pdl_grid(g), v.Axu != v.Ax ? k_resid_scaled<T, true, kFlat> : k_resid_scaled<T, false, kFlat>,
                       grid, 256, 0, s, g, sh, v.Ad, v.Ax, v.Ay, v.Az, v.Axu, v.Ayu, v.Azu, v.b, v.x,
@@ -1021,7 +1030,7 @@ template <class T, bool kFlat>
 cudaError_t apply_impl(const Geo& g, Buffers& b, cudaStream_t s) {
   const Shape sh = shape_of<T, kFlat>(g);
   const IluSet<T> v = set_of(b, (T*)nullptr);
-  const dim3 grid(sh.nty * sh.ntz, (g.nx + kXC<T> - 1) / kXC<T>);
+  const dim3 grid = layout_grid<T>(g, sh);
   count_launches(1);
   return launch_after(pdl_grid(g), k_apply_z<T, kFlat>, grid, 256, 0, s, g, sh, v.z, v.x);
 }

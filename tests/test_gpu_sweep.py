@@ -56,3 +56,28 @@ def test_sweeps_equal_level_schedule(cams, monkeypatch, shape, coarse, precision
         r1, p1 = _iterate(cams, monkeypatch, case, mode)
         assert np.array_equal(p1, p0), mode
         assert np.array_equal(r1, r0), mode
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_a_row_of_more_than_two_million_cells(prec):
+    """65,536 pieces of a row and more in the layout conversions (32 cells a
+    piece in FP64).  On one row A is tridiagonal and ILU(0) is its LU
+    factorisation, so one smoothing step solves the system: the residual falls
+    to rounding (FP32 in the mixed preconditioner, whose residual is then below
+    1e-3 of the first: u times the condition number of D^-1 A, diagonally
+    dominant by dt here)."""
+    from paper_1705_05783_gb300 import cams
+    n = 65535 * 32 + 1000 + 64
+    n -= n % 1000
+    k = np.exp(np.random.default_rng(3).standard_normal(n))
+    h = cams.cams_setup(cams.cams_grid(n, 1, 1, 1.0, 1.0, 1.0), cams.cams_fluid(0, 0.1, 1.0, 1.0, 1.0),
+                        cams.make_options((1000, 1, 1), precision=prec, n_post=1), k)
+    try:
+        bc, keep = cams.make_bc(True, 1.0, 0.0)
+        p0 = np.random.default_rng(4).uniform(0.0, 1.0, n)
+        cams.cams_assemble(h, p0, p0, 1e-2, bc)
+        cams.cams_update_basis(h, True)
+        norms = cams.cams_iterate(h, 1)
+        assert norms[1] <= (1e-3 if prec else 1e-9) * norms[0]
+    finally:
+        cams.cams_destroy(h)
