@@ -6,6 +6,10 @@
 // thread per cell over the x-fastest layout.  Either way every array access
 // of a warp is a coalesced 256-byte run; the neighbour reads of the 7-point
 // stencil hit L1/L2.  FP64 throughout.
+#include <cmath>
+#include <cstdlib>
+#include <limits>
+
 #include "cams_internal.h"
 #include "launch.h"
 #include "rcp64.h"
@@ -27,17 +31,31 @@ __device__ __forceinline__ double rcp_any(double d) {
   return rcp_halley(d);
 }
 
+// Zero, or of a size (2^-460 to 2^460) whose sums, products and reciprocals
+// below neither overflow nor lose digits.
+__device__ __forceinline__ bool moderate(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return (hi >> 20) - 563u <= 920u || (hi | (unsigned)__double2loint(v)) == 0u;
+}
+
 // TPFA: T = A / (h/(2 lambda_a) + h/(2 lambda_b)), as c k_a (k_b / (k_a +
 // k_b)) with c = 2 A / (h mu): one reciprocal a face instead of five
 // divisions, which were the kernel's time (0.97 ms at 4M cells; an FP64
 // division is a chain of about ten FP64 instructions).  Where that is not
-// finite (both permeabilities zero, or out of range) the formula as it stands
-// decides.
+// finite (both permeabilities zero, or c not moderate and given as NaN), or a
+// permeability is not moderate, the formula as it stands decides.
 __device__ __forceinline__ double face_trans(double c, double area, double h, double mu, double ka,
                                              double kb) {
-  const double t = c * (ka * (kb * rcp_any(ka + kb)));
-  if (isfinite(t)) return t;
+  if (moderate(ka) && moderate(kb)) {
+    const double t = c * (ka * (kb * rcp_any(ka + kb)));
+    if (isfinite(t)) return t;
+  }
   return area / (h / (2.0 * (ka / mu)) + h / (2.0 * (kb / mu)));
+}
+// the half cell at a Dirichlet face
+__device__ __forceinline__ double half_trans(double c, double area, double h, double mu, double k) {
+  if (moderate(k) && isfinite(c)) return c * k;
+  return area / (h / (2.0 * (k / mu)));
 }
 
 __global__ void k_transmissibility(Geo g, double mu, const double* __restrict__ kx,
@@ -54,8 +72,8 @@ __global__ void k_transmissibility(Geo g, double mu, const double* __restrict__ 
   Tz[i] = z > 0 ? face_trans(cz, az, g.dz, mu, kz[i - g.sz], kz[i]) : 0.0;
   if (dirichlet) {
     const long long f = y + (long long)g.ny * z;
-    if (x == 0) Tbw[f] = cx * kx[i];
-    if (x == g.nx - 1) Tbe[f] = cx * kx[i];
+    if (x == 0) Tbw[f] = half_trans(cx, ax, g.dx, mu, kx[i]);
+    if (x == g.nx - 1) Tbe[f] = half_trans(cx, ax, g.dx, mu, kx[i]);
   }
 }
 
@@ -351,10 +369,16 @@ inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
 cudaError_t launch_transmissibility(const Geo& g, double mu, const double* kx, const double* ky,
                                     const double* kz, int dirichlet, Buffers& b, cudaStream_t s) {
+  // (a factor that is not moderate, or made from a product that is not, is left
+  // to the formula)
+  auto factor = [&](double a, double d, double h) {
+    const double area = a * d, hm = h * mu, c = 2.0 * area / hm;
+    const auto fits = [](double v) { return std::isnormal(v) && std::abs(std::ilogb(v)) <= 460; };
+    return fits(area) && fits(hm) && fits(c) ? c : std::numeric_limits<double>::quiet_NaN();
+  };
   k_transmissibility<<<blocks_for(g.N, 256), 256, 0, s>>>(
-      g, mu, kx, ky, kz, dirichlet, 2.0 * (g.dy * g.dz) / (g.dx * mu),
-      2.0 * (g.dx * g.dz) / (g.dy * mu), 2.0 * (g.dx * g.dy) / (g.dz * mu), b.Tx, b.Ty, b.Tz,
-      b.Tbw, b.Tbe);
+      g, mu, kx, ky, kz, dirichlet, factor(g.dy, g.dz, g.dx), factor(g.dx, g.dz, g.dy),
+      factor(g.dx, g.dy, g.dz), b.Tx, b.Ty, b.Tz, b.Tbw, b.Tbe);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -159,3 +159,41 @@ def test_a_thin_grid_costs_as_much_as_a_long_one(cams):
             times.append(a.elapsed_time(b))
         return min(times)
     assert best((1, 1, N)) <= 5 * best((N, 1, 1))
+
+
+@pytest.mark.parametrize("mu, dz", [(1e3, 0.5), (1.0, 0.5), (1e-3, 1e-170)])
+def test_transmissibilities_over_the_exponent_range(cams, mu, dz):
+    """The two-point formula as it stands, wherever it is finite, for
+    permeabilities from the smallest normal number to 1.6e308: sums of two that
+    overflow, ratios that underflow.  The formula and the library's form of it are
+    each within five roundings of the exact value (16 eps covers both), as far as
+    the formula's own quotients are normal numbers."""
+    k = np.array([1e-13, 1.0, 3e5, 1e-290, 1e290, 1.6e308, 1.2e308, 1.6e308, 3e-308, 1e200, 1e-200, 1e-13, 1e140, 1e-140,
+                  1e138, 1e308, 1e150, 7.0])
+    nx, h = len(k), (1.0, 0.25, dz)
+    g = cams.cams_grid(nx, 2, 2, *h)
+    kf = np.tile(k, 4)
+    o = cams.make_options((2, 2, 2))
+    hd = cams.cams_setup(g, cams.cams_fluid(0, 0.1, 1.0, mu, 1.0), o, kf)
+    try:
+        T = cams.cams_get(hd, cams.CAMS_Q_TRANS, np.zeros(3 * 4 * nx)).reshape(3, 4 * nx)
+    finally:
+        cams.cams_destroy(hd)
+    eps, tiny = np.finfo(float).eps, np.finfo(float).tiny
+    with np.errstate(all="ignore"):
+        def want(ka, kb, d):
+            area = {0: np.float64(h[1]) * h[2], 1: np.float64(h[0]) * h[2], 2: np.float64(h[0]) * h[1]}[d]
+            qa, qb = h[d] / (2.0 * (ka / mu)), h[d] / (2.0 * (kb / mu))
+            t = area / (qa + qb)
+            ok = np.isfinite(t) & (t >= tiny) & (qa + qb >= tiny)
+            for q, v in ((qa, ka), (qb, kb)):
+                ok &= np.isfinite(q) & (q >= tiny) & np.isfinite(2.0 * (v / mu)) & (v / mu >= tiny)
+            return t, ok
+        i = np.arange(4 * nx)
+        used = 0
+        for d, st, c in ((0, 1, i % nx), (1, nx, i // nx % 2), (2, 2 * nx, i // (2 * nx))):
+            up = i[c > 0]
+            t, ok = want(kf[up - st], kf[up], d)
+            assert np.all(np.abs(T[d][up] - t)[ok] <= 16 * eps * t[ok])
+            used += int(ok.sum())
+    assert used >= 40
