@@ -368,7 +368,12 @@ int cams_surrogate_data(cams_handle* h, int max_patches, float* x, float* target
  *             gbias = dL/dbias and, when gx != NULL, gx = dL/dx multiplied
  *             by the ReLU mask xact > 0 of the layer's input when xact !=
  *             NULL (the gradient with respect to the previous layer's
- *             pre-activation).  gw and gbias are overwritten.
+ *             pre-activation).  gw and gbias are overwritten.  Partial sums
+ *             take a workspace of at most 64 MB, allocated in stream order
+ *             from a pool of the library's that keeps up to that much per
+ *             device between calls (given back by cams_destroy of any
+ *             handle); without it, or on a capturing stream, a slower
+ *             kernel needs none.
  *   mse:      loss = sum(mask (pred - target)^2) / count into *loss (device
  *             double), grad = 2 mask (pred - target) / count; scratch holds
  *             512 doubles.
@@ -458,7 +463,8 @@ int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* diag, const
  * is NULL).  Never NULL; owned by the library. */
 const char* cams_last_error(cams_handle* h);
 
-/* Release every resource of h.  NULL is ignored. */
+/* Release every resource of h, and the device memory that the network's
+ * backward pass keeps between calls.  NULL is ignored. */
 void cams_destroy(cams_handle* h);
 
 #ifdef __cplusplus

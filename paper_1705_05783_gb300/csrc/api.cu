@@ -1886,6 +1886,7 @@ void cams_destroy(cams_handle* h) {
   for (auto& x : h->pool) cudaEventDestroy(x);
   free_all(h);
   delete h;
+  release_net_workspace();
 }
 
 }  // extern "C"

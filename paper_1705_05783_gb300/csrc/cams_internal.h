@@ -213,6 +213,8 @@ cudaError_t launch_adapt_flags(const Geo& g, const Entity* ents, int count, doub
 cudaError_t launch_adapt_propagate(const Geo& g, int first, int count, Buffers& b,
                                    cudaStream_t s);
 cudaError_t launch_count_flags(int count, const unsigned char* flag, double* mail, cudaStream_t s);
+// The current context's number, 0 when it cannot be told (noalloc.cu).
+unsigned long long context_id();
 // Whether kernels on the device can write ordinary host memory (noalloc.cu).
 bool host_writable(int dev);
 // single: P and the local solves in FP32 (mixed precision), else FP64.
@@ -312,6 +314,8 @@ constexpr long long kNetParams = (long long)kNetHid * kNetIn * 27 + kNetHid +
                                  (long long)kNetOut * kNetHid * 27 + kNetOut;
 cudaError_t launch_conv_fwd(int B, int S, int ci, int co, const float* x, const float* w,
                             const float* bias, int relu, float* y, cudaStream_t s);
+// gives the unused memory of launch_conv_bwd's workspace pool back
+void release_net_workspace();
 cudaError_t launch_conv_bwd(int B, int S, int ci, int co, const float* x, const float* w,
                             const float* gy, const float* xact, float* gx, float* gw,
                             float* gbias, cudaStream_t s);

@@ -46,36 +46,12 @@ static_assert(cams::kColBlocks <= kMaxBlocks, "one partial sum per CTA");
 constexpr int kSmallThreads = 1024, kSmallCtas = 8, kSmallPieces = 4 * kSmallCtas;
 constexpr int kMaxDevices = 64;
 
-// cuCtxGetCurrent of the driver API, reached through the runtime (no link
-// against libcuda); its CUcontext is held as an opaque pointer.
-using CtxGetCurrentFn = int (*)(void**);
-
 // partial sums [0, kMaxBlocks) and the total at [kMaxBlocks]
 static __device__ __align__(256) double g_noalloc_scratch[kMaxBlocks + 1];
 
 std::mutex g_mutex;
 double* g_scratch_addr[kMaxDevices] = {};
-void* g_scratch_ctx[kMaxDevices] = {};      // context the address was taken in
-CtxGetCurrentFn g_ctx_get = nullptr;
-bool g_ctx_get_tried = false;
-
-// The calling thread's current context, or null when it cannot be told.
-void* current_context() {
-  if (!g_ctx_get_tried) {
-    g_ctx_get_tried = true;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q{};
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &fn, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      g_ctx_get = reinterpret_cast<CtxGetCurrentFn>(fn);
-    else
-      cudaGetLastError();
-  }
-  void* ctx = nullptr;
-  if (!g_ctx_get || g_ctx_get(&ctx) != 0) return nullptr;
-  return ctx;
-}
+unsigned long long g_scratch_ctx[kMaxDevices] = {};   // context the address was taken in
 
 __global__ void __launch_bounds__(cams::kColThreads) k_residual_noalloc(
     cams::Geo g, cams::ColWork w, const double* __restrict__ Ad, const double* __restrict__ Ax,
@@ -124,6 +100,32 @@ int fail_na(int code, const std::string& msg) {
 
 namespace cams {
 
+// The driver's number of the calling thread's current context, unique in the
+// process (a device's context keeps its handle over cudaDeviceReset, but not its
+// number); 0 when there is none or it cannot be told.  cuCtxGetCurrent and
+// cuCtxGetId are reached through the runtime (no link against libcuda); a
+// CUcontext is held as an opaque pointer.
+unsigned long long context_id() {
+  using GetCurrent = int (*)(void**);
+  using GetId = int (*)(void*, unsigned long long*);
+  static const auto entry = [](const char* name) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q{};
+    if (cudaGetDriverEntryPointByVersion(name, &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return fn;
+  };
+  static const auto get = reinterpret_cast<GetCurrent>(entry("cuCtxGetCurrent"));
+  static const auto id_of = reinterpret_cast<GetId>(entry("cuCtxGetId"));
+  void* ctx = nullptr;
+  unsigned long long id = 0;
+  if (!get || !id_of || get(&ctx) != 0 || !ctx || id_of(ctx, &id) != 0) return 0;
+  return id;
+}
+
 // Whether kernels on the device can write ordinary host memory.
 bool host_writable(int dev) {
   static std::atomic<int> known[kMaxDevices];   // 0 not asked, 1 no, 2 yes
@@ -162,13 +164,13 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
   {
     // set-up, once per device and context, with that device current
     std::lock_guard<std::mutex> lock(g_mutex);
-    void* ctx = current_context();
+    const unsigned long long ctx = cams::context_id();
     if (!g_scratch_addr[dev] || !ctx || ctx != g_scratch_ctx[dev]) {
       e = cudaGetSymbolAddress(reinterpret_cast<void**>(&scratch), g_noalloc_scratch);
       if (e != cudaSuccess)
         return fail_na(CAMS_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
       g_scratch_addr[dev] = scratch;
-      g_scratch_ctx[dev] = current_context();   // the lookup made the primary context current
+      g_scratch_ctx[dev] = cams::context_id();   // the lookup made the primary context current
     }
     scratch = g_scratch_addr[dev];
   }
