@@ -783,16 +783,29 @@ void release_net_workspace() {
 namespace {
 constexpr int kSms = 152;               // SMs of the GPU
 constexpr int kTileSmem = 100 * 1024;   // more leaves one CTA per SM: the general kernels then
+constexpr int kFewCi = 260;             // summed channels whose weights fit a general kernel's CTA
 }  // namespace
 
-// The tiled kernel wherever a CTA's planes fit its staging (every patch up to
-// 24^3 or so), else the general one.  64 patches of 11^3: 32 -> 32 channels
-// 390 -> 176 us, 32 -> 8 channels 132 -> 79.
+// Warps that the general kernels would run for `c` result channels.  Where they
+// are few, one CTA's latency is the time whatever the batch, and the general
+// kernels' is the shorter (8 channels a CTA instead of 32).
+static long long general_warps(int B, int S, int c) {
+  return (long long)B * ((c + kCoB - 1) / kCoB) * (((long long)S * S * S + 31) / 32);
+}
+
+// The tiled kernel where a CTA's planes fit its staging (with the strips per CTA
+// that the batch's size gives it: most patches up to 12^3, few above), else the
+// general one.  64 patches of 11^3: 32 -> 32 channels 390 -> 176 us, 32 -> 8
+// channels 132 -> 79.  With 8 results a thread the general kernel is the faster
+// one up to 1024 warps of its own (32 -> 32, 64 patches of 4^3: 72 against 78 us; 64 of
+// 6^3, beyond the line: 91 against 74); so it is for patches of one voxel.
 cudaError_t launch_conv_fwd(int B, int S, int ci, int co, const float* x, const float* w,
                             const float* bias, int relu, float* y, cudaStream_t s) {
   const int S3 = S * S * S;
   const ConvTile t = conv_tile(B, S, co, kSms);
-  if (t.smem <= kTileSmem) {
+  const int smem = kCoB * ci * 27 * (int)sizeof(float);
+  const bool few = S == 1 || (t.ko == 8 && general_warps(B, S, co) <= 1024);
+  if (t.smem <= kTileSmem && !(few && ci <= kFewCi)) {
     cudaError_t e = t.ko == 8 ? raise_smem_limit(k_conv_tile<false, 8>, t.smem)
                                 : raise_smem_limit(k_conv_tile<false, 4>, t.smem);
     if (e != cudaSuccess) return e;
@@ -802,7 +815,6 @@ cudaError_t launch_conv_fwd(int B, int S, int ci, int co, const float* x, const 
     count_launches(1);
     return cudaGetLastError();
   }
-  const int smem = kCoB * ci * 27 * (int)sizeof(float);
   cudaError_t e = raise_smem_limit(k_conv_fwd, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((S3 + kNetThreads * kVox - 1) / (kNetThreads * kVox), (co + kCoB - 1) / kCoB, B);
@@ -816,6 +828,11 @@ cudaError_t launch_conv_fwd(int B, int S, int ci, int co, const float* x, const 
 // The general weight kernel stays for patches whose planes do not fit and for
 // a stream that is being captured (a graph would have to own the workspace).
 // 64 patches of 11^3, 32 x 32 channels: data 440 -> 174 us, weights 1400 -> 180.
+// Small calls stay with the general kernels here too: the data gradient up to 2048
+// of their warps where 16 channels or fewer are summed (8 channels, 64 patches of
+// 4^3: 31 against 37 us; of 8^3, beyond the line: 53 against 37), and the weights where a CTA
+// per pair of channels has few passes of 256 voxels to make (4 patches of 11^3,
+// 32 x 8 channels: 33 against 21 us; 1 patch: 13 against 19).
 cudaError_t launch_conv_bwd(int B, int S, int ci, int co, const float* x, const float* w,
                             const float* gy, const float* xact, float* gx, float* gw,
                             float* gbias, cudaStream_t s) {
@@ -823,13 +840,14 @@ cudaError_t launch_conv_bwd(int B, int S, int ci, int co, const float* x, const 
   cudaError_t e;
   if (gx) {
     const ConvTile t = conv_tile(B, S, ci, kSms);
-    if (t.smem <= kTileSmem) {
+    const bool few = S == 1 || (t.ko == 8 && co <= 16 && general_warps(B, S, ci) <= 2048);
+    if (t.smem <= kTileSmem && !(few && co <= kFewCi)) {
       e = t.ko == 8 ? raise_smem_limit(k_conv_tile<true, 8>, t.smem)
                                 : raise_smem_limit(k_conv_tile<true, 4>, t.smem);
       if (e != cudaSuccess) return e;
       dim3 grid((S * t.NYP * t.NS + t.ST - 1) / t.ST, (ci + 31) / 32, B);
       if (t.ko == 8) k_conv_tile<true, 8><<<grid, t.ST * t.ncg, t.smem, s>>>(S, co, ci, t, gy, w, nullptr, 0, xact, gx);
-    else k_conv_tile<true, 4><<<grid, t.ST * t.ncg, t.smem, s>>>(S, co, ci, t, gy, w, nullptr, 0, xact, gx);
+      else k_conv_tile<true, 4><<<grid, t.ST * t.ncg, t.smem, s>>>(S, co, ci, t, gy, w, nullptr, 0, xact, gx);
     } else {
       const int smem = kCoB * co * 27 * (int)sizeof(float);
       e = raise_smem_limit(k_conv_bwd_data, smem);
@@ -850,7 +868,9 @@ cudaError_t launch_conv_bwd(int B, int S, int ci, int co, const float* x, const 
     cudaGetLastError();
     cap = cudaStreamCaptureStatusActive;
   }
-  if (smem <= kTileSmem && cap == cudaStreamCaptureStatusNone) {
+  const long long passes = (long long)B * (((long long)S * S * S + 255) / 256);
+  const bool few = passes * (1024 + (long long)ci * co) < 20 * 1024;
+  if (smem <= kTileSmem && cap == cudaStreamCaptureStatusNone && !few) {
     // chunks: of one plane at least, and as many as the workspace holds (with many
     // channels the tiles fill the chip, whatever the chunks)
     const long long units = (long long)B * S, per = (long long)co * ci * 27 + co;
