@@ -49,3 +49,57 @@ def test_which_kernels_a_weight_gradient_takes(env, B, S, ci, co, kernels):  # n
         assert cams.cams_get(h, cams.CAMS_Q_LAUNCHES, np.zeros(1))[0] - n0 == kernels
     finally:
         cams.cams_destroy(h)
+
+
+@pytest.mark.parametrize("what", ["an inf", "all nan", "nan weights"])
+def test_non_finite_inputs_take_no_longer_than_without_tiles(env, what):  # noqa: F811
+    """A sum that padding or a zero gradient may have made non-finite is formed again
+    by a whole CTA: the call stays within three times its time on finite inputs
+    plus the general kernel's 1.4 ms (ten times that with a thread a sum), and
+    what is non-finite is what FP64 makes non-finite from the pairs of voxels
+    inside the patch with a gradient."""
+    torch, cams = env
+    B, S, ci, co = 64, 11, 32, 32
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(B, ci, S, S, S, generator=g, device="cuda")
+    w = torch.randn(co, ci, 27, generator=g, device="cuda")
+    gy = torch.randn(B, co, S, S, S, generator=g, device="cuda")
+    gy[:, :, 0, 0, :3] = 0.0
+    gw, gb, gx = torch.zeros_like(w), torch.zeros(co, device="cuda"), torch.zeros_like(x)
+
+    def best():
+        ts = []
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            cams.cams_net_conv_backward(B, S, ci, co, x, w, gy, None, gx, gw, gb)
+            b.record()
+            b.synchronize()
+            ts.append(a.elapsed_time(b))
+        return min(ts)
+    base = best()
+    finite = gw.clone()
+    if what == "an inf":
+        x[5, 7, 0, 0, 0] = float("inf")
+        # g is zero at the voxel itself and beside it along x: those two taps stay as they were
+        # (dx = 0 and -1 of dy = dz = 0), other channels too; others see the infinity
+        want = torch.zeros(co, ci, 27, dtype=torch.bool, device="cuda")
+        for t in range(27):
+            dx, dy, dz = t % 3 - 1, t // 3 % 3 - 1, t // 9 - 1
+            if dx <= 0 and dy <= 0 and dz <= 0 and not (dy == 0 and dz == 0):
+                want[:, 7, t] = True
+    elif what == "all nan":
+        x[:] = float("nan")
+        want = torch.ones(co, ci, 27, dtype=torch.bool, device="cuda")
+    else:
+        w[:] = float("nan")
+        want = torch.zeros(co, ci, 27, dtype=torch.bool, device="cuda")
+    t = best()
+    assert bool((torch.isfinite(gw) != want).all())
+    if what == "an inf":
+        rest = ~want
+        rest[:, 7] = False
+        assert torch.equal(gw[rest], finite[rest])
+        assert bool(((gw - finite).abs() <= 2 * B * S ** 3 * U * 64.0)[~want].all())
+    assert bool(torch.isnan(gx).all()) == (what == "nan weights")
+    assert t <= 3 * base + 1.4
