@@ -972,7 +972,10 @@ cudaError_t run_sweep(const Geo& g, const Shape& sh, const IluSet<T>& v, bool ct
   // 8 CTAs a cluster (the portable limit).  Measured at 200 x 200 x 100, FP32 /
   // FP64: 2 x 4 tiles 98 / 145 us, 4 x 2 98 / 147, 8 x 1 118 / 159, 1 x 8
   // 159 / 199, no clusters 122 / 188 (hand-overs through L2 only).
-  const int nbz = !cta || kFlat ? 1 : sh.ntz >= 4 ? 4 : 2, nby = cta ? 8 / nbz : 1;
+  // A grid of one row of tiles takes its clusters along it: half of their CTAs
+  // would have no tile, and be counted in the hand-overs (1 x 1 x 20000, FP32: a
+  // sweep of 8.7 ms with 2 x 4, 4.4 with 1 x 8; 300 x 300 x 3: 74 and 70 us).
+  const int nbz = !cta || kFlat || sh.ntz == 1 ? 1 : sh.nty == 1 ? 8 : sh.ntz >= 4 ? 4 : 2, nby = cta ? 8 / nbz : 1;
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3((unsigned)(sweep_clusters<T, kFlat>(sh, nby, nbz) * nby * nbz));
   c.blockDim = dim3(Pl::kThreads);

@@ -81,3 +81,11 @@ def test_a_row_of_more_than_two_million_cells(prec):
         assert norms[1] <= (1e-3 if prec else 1e-9) * norms[0]
     finally:
         cams.cams_destroy(h)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("shape,coarse", [((5, 8, 90), (5, 4, 9)),     # one tile wide in y: clusters along z
+                                          ((30, 150, 4), (5, 10, 2)),  # ... in z: clusters along y
+                                          ((560, 3, 34), (8, 3, 17))]) # rows longer than the rings, one tile wide
+def test_sweeps_of_one_row_of_tiles(cams, monkeypatch, shape, coarse, precision):
+    test_sweeps_equal_level_schedule(cams, monkeypatch, shape, coarse, precision)
