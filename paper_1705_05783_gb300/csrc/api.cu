@@ -1179,10 +1179,13 @@ int cams_setup(const cams_grid* grid, const cams_fluid* fluid, const cams_option
     h->ilu_pipelined = !(lv && lv[0] == '1');
     h->sms = prop.multiProcessorCount;
     // blocks of tiles per cluster; CAMS_ILU_CTA=0 runs every tile on its own
+    // (where their shared memory does not fit, the level schedule, which needs none)
     const char* ct = std::getenv("CAMS_ILU_CTA");
-    ilu_set_smem();
-    ilu_sweep_smem((int)prop.sharedMemPerBlockOptin);
-    h->ilu_cta = !(ct && ct[0] == '0');
+    if (!ilu_set_smem() || !ilu_sweep_smem((int)prop.sharedMemPerBlockOptin)) {
+      cudaGetLastError();
+      h->ilu_pipelined = false;
+    }
+    h->ilu_cta = h->ilu_pipelined && !(ct && ct[0] == '0');
     const char* cc = std::getenv("CAMS_COARSE_CLUSTER");
     h->coarse_cluster = !(cc && cc[0] == '0') &&
                         coarse_cluster_ok(h->c.Nc, (int)prop.sharedMemPerBlockOptin);
