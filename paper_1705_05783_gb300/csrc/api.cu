@@ -1185,7 +1185,7 @@ int cams_setup(const cams_grid* grid, const cams_fluid* fluid, const cams_option
       cudaGetLastError();
       h->ilu_pipelined = false;
     }
-    h->ilu_cta = h->ilu_pipelined && !(ct && ct[0] == '0');
+    h->ilu_cta = h->ilu_pipelined && !(ct && ct[0] == '0') && ilu_cluster_ok(h->g, h->single);
     const char* cc = std::getenv("CAMS_COARSE_CLUSTER");
     h->coarse_cluster = !(cc && cc[0] == '0') &&
                         coarse_cluster_ok(h->c.Nc, (int)prop.sharedMemPerBlockOptin);
@@ -1306,6 +1306,8 @@ int cams_set_schedule(cams_handle* h, int ilu_cta, int coarse_cluster) {
     return fail(h, CAMS_EINVAL, "the level-scheduled sweeps have no tile schedule");
   cudaDeviceProp prop;
   CK(cudaGetDeviceProperties(&prop, h->dev));
+  if (ilu_cta == 1 && !h->ilu_cta && !ilu_cluster_ok(h->g, h->single))
+    return fail(h, CAMS_EINVAL, "blocks of tiles per cluster are not available on this device");
   if (coarse_cluster == 1 && !h->coarse_cluster &&
       !coarse_cluster_ok(h->c.Nc, (int)prop.sharedMemPerBlockOptin))
     return fail(h, CAMS_EINVAL, "the cluster coarse solve is not available for this coarse grid");

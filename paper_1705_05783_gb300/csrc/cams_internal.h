@@ -300,6 +300,8 @@ cudaError_t launch_ilu_apply(const Geo& g, Buffers& b, bool single, cudaStream_t
 // raise the kernels' shared-memory limits; false when one does not fit
 bool ilu_set_smem();
 bool ilu_sweep_smem(int max_smem);
+// whether the sweeps' clusters can be resident
+bool ilu_cluster_ok(const Geo& g, bool single);
 cudaError_t launch_add_correction(const Geo& g, Buffers& b, cudaStream_t s);   // p += delta
 int ilu_ctrl_ints(const Geo& g);
 // Rows per factorisation tile (y, z), and the length of a sweep vector.

@@ -2267,9 +2267,13 @@ static int coarse_twist_smem(const Twist& tw, int bytes = 8) {
 }
 
 bool coarse_twist_ok(const Twist& tw, int max_smem) {
-  return tw.H > 0 && coarse_twist_smem(tw) <= max_smem &&
-         raise_smem_limit(k_coarse_solve_twisted<double>, coarse_twist_smem(tw)) == cudaSuccess &&
-         raise_smem_limit(k_coarse_solve_twisted<float>, coarse_twist_smem(tw, 4)) == cudaSuccess;
+  if (tw.H == 0 || coarse_twist_smem(tw) > max_smem) return false;
+  if (raise_smem_limit(k_coarse_solve_twisted<double>, coarse_twist_smem(tw)) != cudaSuccess ||
+      raise_smem_limit(k_coarse_solve_twisted<float>, coarse_twist_smem(tw, 4)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cluster_fits(k_coarse_solve_twisted<double>, kCC, 256, coarse_twist_smem(tw));
 }
 
 bool coarse_cluster_ok(int Nc, int max_smem) {
@@ -2280,21 +2284,7 @@ bool coarse_cluster_ok(int Nc, int max_smem) {
     cudaGetLastError();
     return false;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCC);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCC;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_coarse_solve_cluster<double>, &cfg) != cudaSuccess) n = 0;
-  cudaGetLastError();
-  return n > 0;
+  return cluster_fits(k_coarse_solve_cluster<double>, kCC, 256, smem);
 }
 
 cudaError_t launch_band_solve(const Geo& g, int Nc, int m, int sym, bool cluster, bool single,

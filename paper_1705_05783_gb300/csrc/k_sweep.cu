@@ -69,6 +69,7 @@ constexpr int kSlots = 8;                    // operand slots: steps staged ahea
 constexpr int kTeam = 4;                     // warps per tile
 constexpr long long kPollLimit = 1LL << 22;  // helper polls without progress before a wait gives up
 constexpr long long kSpinLimit = 1LL << 26;  // shared-memory polls before a wait gives up
+constexpr int kSweepCtas = 8;                // CTAs of a cluster
 constexpr int kSpare = kStep;                // spare records at both ends of a vector
 
 // A chunk of G cells of one row, and the "not computed yet" sentinel: a
@@ -975,7 +976,8 @@ cudaError_t run_sweep(const Geo& g, const Shape& sh, const IluSet<T>& v, bool ct
   // A grid of one row of tiles takes its clusters along it: half of their CTAs
   // would have no tile, and be counted in the hand-overs (1 x 1 x 20000, FP32: a
   // sweep of 8.7 ms with 2 x 4, 4.4 with 1 x 8; 300 x 300 x 3: 74 and 70 us).
-  const int nbz = !cta || kFlat || sh.ntz == 1 ? 1 : sh.nty == 1 ? 8 : sh.ntz >= 4 ? 4 : 2, nby = cta ? 8 / nbz : 1;
+  const int nbz = !cta || kFlat || sh.ntz == 1 ? 1 : sh.nty == 1 ? 8 : sh.ntz >= 4 ? 4 : 2;
+  const int nby = cta ? kSweepCtas / nbz : 1;
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3((unsigned)(sweep_clusters<T, kFlat>(sh, nby, nbz) * nby * nbz));
   c.blockDim = dim3(Pl::kThreads);
@@ -1064,6 +1066,12 @@ bool allow_smem(int max_smem) {
          raise_smem_limit(k_sweep<T, true, kFlat>, bytes) == cudaSuccess;
 }
 
+template <class T, bool kFlat>
+bool cluster_ok() {
+  return cluster_fits(k_sweep<T, false, kFlat>, kSweepCtas, Plan<T, kFlat>::kThreads, Plan<T, kFlat>::kBytes) &&
+         cluster_fits(k_sweep<T, true, kFlat>, kSweepCtas, Plan<T, kFlat>::kThreads, Plan<T, kFlat>::kBytes);
+}
+
 }  // namespace
 
 namespace {
@@ -1084,6 +1092,8 @@ bool ilu_sweep_smem(int max_smem) {
 #define CAMS_BY_SHAPE(fn, ...)                                                       \
   (single ? (g.nz == 1 ? fn<float, true>(__VA_ARGS__) : fn<float, false>(__VA_ARGS__)) \
           : (g.nz == 1 ? fn<double, true>(__VA_ARGS__) : fn<double, false>(__VA_ARGS__)))
+
+bool ilu_cluster_ok(const Geo& g, bool single) { return CAMS_BY_SHAPE(cluster_ok); }
 
 long long ilu_sweep_len(const Geo& g, bool single) { return CAMS_BY_SHAPE(sweep_len, g); }
 

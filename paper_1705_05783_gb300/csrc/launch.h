@@ -29,6 +29,26 @@ inline cudaLaunchAttribute pdl_attribute() {
   return a;
 }
 
+// Whether the device can hold a cluster of `ctas` such CTAs at all (a part of it
+// may not: a partition, a limit on its SMs).
+template <class... P>
+bool cluster_fits(void (*kern)(P...), int ctas, int threads, int smem) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)ctas);
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = (size_t)smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &c) != cudaSuccess) n = 0;
+  cudaGetLastError();
+  return n > 0;
+}
+
 template <class... P, class... A>
 cudaError_t launch_after(bool pdl, void (*kern)(P...), dim3 grid, int threads, int smem, cudaStream_t s,
                          A&&... args) {

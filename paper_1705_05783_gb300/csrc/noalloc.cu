@@ -91,6 +91,17 @@ __global__ void k_finish_noalloc(int nblocks, const double* scratch, double* tot
   if (threadIdx.x == 0) *total = s;
 }
 
+// Whether the device can hold k_residual_small's clusters (asked once).
+bool small_fits(int dev) {
+  static std::atomic<int> known[kMaxDevices];   // 0 not asked, 1 no, 2 yes
+  int k = known[dev].load(std::memory_order_relaxed);
+  if (k == 0) {
+    k = cams::cluster_fits(k_residual_small, kSmallCtas, kSmallThreads, 0) ? 2 : 1;
+    known[dev].store(k, std::memory_order_relaxed);
+  }
+  return k == 2;
+}
+
 int fail_na(int code, const std::string& msg) {
   cams::set_global_error(msg);
   return code;
@@ -189,7 +200,7 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
   double* total = direct ? &s2 : scratch + kMaxBlocks;
   const char* what = "launch: ";
   cams::ColWork w = cams::col_work(g, kSmallThreads);
-  if (w.pieces <= (unsigned)kSmallPieces) {
+  if (w.pieces <= (unsigned)kSmallPieces && small_fits(dev)) {
     int ctas = 1;
     while (ctas < kSmallCtas && ctas < (int)w.pieces) ctas *= 2;
     cudaLaunchConfig_t cfg{};
