@@ -147,15 +147,20 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(int B, TcGeom G, int ci,
   bool ok = true;
   if (warp == 5) {
     if ((t & 31) == 0) {
-      uint32_t phase = 0;
+      uint32_t phase = 0, last = 0;
+      bool issued = false;
       for (int b = blockIdx.x; b < B && ok; b += gridDim.x, phase ^= 1u) {
         // (a new barrier's preceding phase counts as complete)
         ok = tc::mbar_wait(empty, phase ^ 1u, kTcWait);
         if (ok) {
           tc::mbar_arrive_expect_tx(full, (uint32_t)xbytes);
           tc::bulk_g2s(xs, x + (long long)b * KCin * G.RP * 8, (uint32_t)xbytes, full);
+          issued = true;
+          last = phase;
         }
       }
+      // the CTA does not end with a copy in flight, whoever gave up on it
+      if (issued && !tc::mbar_wait(full, last, kTcWait)) ok = false;
     }
   } else if (warp == 4) {
     if ((t & 31) == 0) {
@@ -188,6 +193,8 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(int B, TcGeom G, int ci,
           if (m == G.nt - 1) tc::mma_commit(empty);
         }
       }
+      // ... nor with MMAs in flight (the read-back may have given up on them)
+      if (!ok && it > 0) tc::mbar_wait(done + ((it - 1) & 1), (uint32_t)((it - 1) >> 1 & 1), kTcWait);
     }
   } else {
     int it = 0;
