@@ -197,3 +197,28 @@ def test_transmissibilities_over_the_exponent_range(cams, mu, dz):
             assert np.all(np.abs(T[d][up] - t)[ok] <= 16 * eps * t[ok])
             used += int(ok.sum())
     assert used >= 40
+
+
+def test_transmissibilities_are_correctly_rounded(cams):
+    """T = 2 A k_a k_b / (h mu (k_a + k_b)) to one rounding, u = 2^-53: numerator,
+    denominator and the quotient's remainder carry their rounding errors, so what is
+    left beside the last rounding is of the order of u^2 (a hundredth of u here)."""
+    nx, ny, nz, h, mu = 45, 34, 23, (0.3, 1.7, 0.9), 0.77
+    N = nx * ny * nz
+    k = np.exp(3.0 * np.random.default_rng(8).standard_normal(N))
+    k[::97] *= 1e40
+    hd = cams.cams_setup(cams.cams_grid(nx, ny, nz, *h), cams.cams_fluid(0, 0.1, 1.0, mu, 1.0),
+                         cams.make_options((5, 2, 23)), k)
+    try:
+        T = cams.cams_get(hd, cams.CAMS_Q_TRANS, np.zeros(3 * N)).reshape(3, N)
+    finally:
+        cams.cams_destroy(hd)
+    Q = np.longdouble
+    assert np.finfo(Q).eps <= 2.0 ** -60
+    i = np.arange(N)
+    for d, st, c in ((0, 1, i % nx), (1, nx, i // nx % ny), (2, nx * ny, i // (nx * ny))):
+        up = i[c > 0]
+        ka, kb = k[up - st].astype(Q), k[up].astype(Q)
+        area = Q(h[0]) * Q(h[1]) * Q(h[2]) / Q(h[d])
+        t = 2 * area * ka * kb / (Q(h[d]) * Q(mu) * (ka + kb))
+        assert float((np.abs(T[d][up] - t) / t).max()) <= 1.01 * 2.0 ** -53
