@@ -59,25 +59,32 @@ BYTES_PER_CELL = {
     "ilu_factor": 88,          # A x4 -> 1/d, scaled couplings x6
     "basis_op": 64,
 }
-# Latency model of a wavefront sweep: its last cell is (nx + ny + nz - 3)
-# dependent steps after its first, so no schedule finishes before that many
-# steps of one tile's step loop.  T_STEP_US: a tile's time per step alone
-# (no neighbour to wait for), measured on this GPU with a lone 8 x 4-row
-# tile of 65,536 x-positions (one group of 4 steps: 0.30 us in FP32,
-# 0.78 us in FP64).
-T_STEP_US = {0: 0.78 / 4, 1: 0.30 / 4}
+# Latency model of a wavefront sweep: a lane's step is a chunk of CHUNK cells of
+# its row, and the sweep's last chunk is (nx / CHUNK + ny + nz - 3) dependent
+# steps after its first.  T_STEP_US: a tile's time per step alone (no neighbour to
+# wait for), measured on this GPU with a lone 8 x 4-row tile of 65,536
+# x-positions (9.40 ms in FP64, 1.80 in FP32): what these kernels take on that
+# chain with hand-overs that cost nothing.
+CHUNK = {0: 1, 1: 4}
+T_STEP_US = {0: 0.1435, 1: 0.110}
 SWEEP_CLASSES = ("ilu_fwd", "ilu_bwd")
 
 # DRAM bytes per launch measured by ncu (dram__bytes_read.sum + write.sum) for
-# a kernel class on a workload; see profiles/.  (Measured with the sweeps of one
-# tile a warp; the cluster sweeps read and write the same operands:
-# profiles/launch_list_3d-200x200x100-mixed-clusters.md.)
+# a kernel class on a workload, of the sweeps of one tile a warp that ran before
+# the cluster sweeps: a record (profiles/launch_list_3d-200x200x100-mixed.md).
 MEASURED_TRAFFIC = {
-    # profiles/launch_list_3d-200x200x100-mixed.md (the kernels as of the FP32 residual copy)
     ("3d-200x200x100-mixed", "ilu_fwd"): 73.9e6,
     ("3d-200x200x100-mixed", "ilu_bwd"): 70.1e6,
     ("3d-200x200x100-mixed", "ilu_resid"): 121.9e6,
     ("3d-200x200x100-mixed", "ilu_apply"): 32.8e6,
+}
+# The same of the present kernels, which the bench line reports
+# (profiles/launch_list_3d-200x200x100-mixed-clusters.md).
+CLUSTER_TRAFFIC = {
+    ("3d-200x200x100-mixed", "ilu_fwd"): 87.6e6,
+    ("3d-200x200x100-mixed", "ilu_bwd"): 84.0e6,
+    ("3d-200x200x100-mixed", "ilu_resid"): 125.5e6,
+    ("3d-200x200x100-mixed", "ilu_apply"): 34.2e6,
 }
 
 # the same classes with the FP32 preconditioner (4-byte operands; r and p stay FP64)
@@ -205,14 +212,13 @@ def class_rooflines(prof, n_cells, precision, peak):
 
 
 def sweep_latency_bound(prof, w):
-    """The ILU(0) sweeps against their critical path: (nx + ny + nz - 3)
-    steps at a lone tile's step time (a bound no schedule of the exact
-    lexicographic recurrence beats at that step time)."""
-    steps = w.nx + w.ny + w.nz - 3
-    bound_us = steps * T_STEP_US[1 if w.precision else 0]
-    out = {"model": "(nx+ny+nz-3) dependent steps x t_step of a lone tile",
-           "t_step_us": T_STEP_US[1 if w.precision else 0], "steps": steps,
-           "bound_us": bound_us}
+    """The ILU(0) sweeps against their chain of dependent steps, of CHUNK cells
+    each, at a lone tile's step time: what hand-overs between tiles add is the rest."""
+    mixed = 1 if w.precision else 0
+    steps = -(-w.nx // CHUNK[mixed]) + w.ny + w.nz - 3
+    bound_us = steps * T_STEP_US[mixed]
+    out = {"model": f"(nx/{CHUNK[mixed]}+ny+nz-3) dependent steps x t_step of a lone tile",
+           "t_step_us": T_STEP_US[mixed], "steps": steps, "bound_us": bound_us}
     for k in SWEEP_CLASSES:
         if k in prof and prof[k][0]:
             avg_us = 1e3 * prof[k][1] / prof[k][0]
@@ -431,7 +437,7 @@ def run_cams(args, w, rank, world, local_rank, e2e_leg=True, surrogate=None):
         "kernel_ms_per_step": {k: v[1] / args.steps for k, v in prof.items() if v[0]},
         "roofline": {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_kind,
-                     "traffic": MEASURED_TRAFFIC.get((w.name, dom)),
+                     "traffic": CLUSTER_TRAFFIC.get((w.name, dom)),
                      "bytes_per_launch": bytes_per_launch,
                      "avg_launch_ms": avg_ms,
                      "timing": "CUDA events per kernel class on the handle's stream, in a "

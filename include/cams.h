@@ -434,12 +434,10 @@ int cams_get_int(cams_handle* h, int what, int* dst);
  * all device memory to their own pool or arena (an allocation behind the
  * pool's back can fail or fragment it) and time-critical loops that cannot
  * afford the device-wide synchronisation cudaMalloc/cudaFree imply.  The
- * reduction's scratch is a file-scope static device array of 32769 doubles
- * (256 KiB), present on every GPU that loads the library until the process
- * exits.
+ * reduction's scratch is a file-scope static device array of 913 doubles,
+ * present on every GPU that loads the library until the process exits.
  *   nx, ny, nz       grid (cell i = x + nx*(y + ny*z)); at most 268,435,456
- *                    cells (32768 partial sums of 8192 cells), else
- *                    CAMS_EINVAL with a message naming the limit
+ *                    cells, else CAMS_EINVAL with a message naming the limit
  *   diag, ax, ay, az A in the CAMS_Q_MATRIX layout (diagonal, then the
  *                    couplings a_{i,i-1}, a_{i,i-nx}, a_{i,i-nx*ny}, stored
  *                    at the upper cell, 0 where absent); DEVICE pointers

@@ -1584,9 +1584,6 @@ int cams_set_surrogate(cams_handle* h, const float* params, double gate_tol) {
     if (!rc) rc = dalloc(h, &tb, n);
     h->surr_ta = ta;
     h->surr_tb = tb;
-    // rows outside the output-tile range are never written: they hold the zero border
-    if (!rc && (cudaMemset(ta, 0, 2 * n) != cudaSuccess || cudaMemset(tb, 0, 2 * n) != cudaSuccess))
-      rc = fail(h, CAMS_ECUDA, "cudaMemset failed");
   } else {
     if (!rc) rc = dalloc(h, &h->surr_h1, (size_t)(h->surr_chunk * kNetHid * S3));
     if (!rc) rc = dalloc(h, &h->surr_h2, (size_t)(h->surr_chunk * kNetHid * S3));

@@ -20,8 +20,8 @@
 // 16 columns x 8 right-hand sides, one thread each, the next panel copied
 // ahead (cp.async).
 //
-// What bounds it: in FP64 the FP64 unit (73% busy; a warp instruction holds it
-// for about 64 cycles, so lanes without work cost as much as others), in FP32
+// What bounds it: in FP64 the FP64 unit (91% busy on 9^3 interiors, 73% on 9 x 9 x 4;
+// a warp instruction holds it for about 64 cycles, so lanes without work cost as much as others), in FP32
 // the instructions issued (66% of the cycles).  The right-looking kernel
 // (k_basis.cu) reads and writes the whole trailing window in shared memory for
 // every 8 pivots, divides in the pivots' chain, and leaves half of the FP64

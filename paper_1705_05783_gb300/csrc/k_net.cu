@@ -189,8 +189,9 @@ __global__ void __launch_bounds__(kNetThreads) k_conv_bwd_w(int B, int S, int ci
 // of results and every value read from shared memory feeds several of them;
 // inputs are staged zero-padded, rows cut into strips of 4 voxels, so the inner
 // loops have no conditions, and two FMAs go in one instruction.  What bounds
-// them then is how many warps a CTA's registers and staging leave (the kernels
-// issue in 0.6 of the cycles with 10 warps an SM), next the FP32 rate: 2.4e9
+// them then is how many warps a CTA's registers and staging leave (9 an SM in the
+// convolutions, which issue in 0.40 to 0.42 of the cycles, 13 in the weight
+// gradient, 0.57), next the FP32 rate: 2.4e9
 // FMAs of 32 x 32 channels on 64 patches of 11^3 take 60 us at it.
 constexpr int kStrip = 4;      // voxels of a strip (one 16-byte read)
 constexpr int kCiB = 4;        // input channels staged at a time (two stages in flight)

@@ -5,7 +5,7 @@
 // fragment it), and time-critical loops that must not pay the device-wide
 // synchronisation that cudaMalloc/cudaFree imply.  This entry point serves
 // them: the caller passes the system and the output buffers, and the
-// reduction's scratch (one partial sum per block of cells plus the total)
+// reduction's scratch (one partial sum per CTA plus the total)
 // lives in a file-scope static device array instead of a handle allocation.
 //
 // The array exists once per device that loads the library and stays there
@@ -32,22 +32,20 @@
 
 namespace {
 
-constexpr int kCellsPerBlock = 8192;    // the largest grid is kMaxBlocks times this
-constexpr int kMaxBlocks = 32768;       // partial sums the scratch holds (256 KiB)
-constexpr long long kMaxCells = (long long)kCellsPerBlock * kMaxBlocks;   // 268,435,456
-static_assert(cams::kColBlocks <= kMaxBlocks, "one partial sum per CTA");
+// the entry point's limit, part of its contract (no buffer here depends on it)
+constexpr long long kMaxCells = 1LL << 28;   // 268,435,456
 
 // A grid of at most kSmallPieces pieces of kSmallThreads columns goes to one
 // cluster, whose CTAs sum up through distributed shared memory: the second
 // launch that adds the partial sums would cost as much as the residual.  (A
-// call on 40 x 40 cells: 19 us, of which 6 are the caller's Python; 36 with
-// two launches and a copy of the total.  On 32 x 32 x 32 cells, the largest of
-// the rule, 26 against 29.)
+// call on 40 x 40 cells: 23 us, of which 6 are the caller's Python; 36 with two
+// launches and a copy of the total.  On 32 x 32 x 32 cells, the largest of the
+// rule, 26 against 29.)
 constexpr int kSmallThreads = 1024, kSmallCtas = 8, kSmallPieces = 4 * kSmallCtas;
 constexpr int kMaxDevices = 64;
 
-// partial sums [0, kMaxBlocks) and the total at [kMaxBlocks]
-static __device__ __align__(256) double g_noalloc_scratch[kMaxBlocks + 1];
+// one partial sum per CTA, then the total
+static __device__ __align__(256) double g_noalloc_scratch[cams::kColBlocks + 1];
 
 std::mutex g_mutex;
 double* g_scratch_addr[kMaxDevices] = {};
@@ -162,9 +160,7 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
   if (N > kMaxCells)
     return fail_na(CAMS_EINVAL, "cams_residual_norm_noalloc: the grid has " + std::to_string(N) +
                                     " cells; at most " + std::to_string(kMaxCells) +
-                                    " are supported (the static scratch holds " +
-                                    std::to_string(kMaxBlocks) + " partial sums of " +
-                                    std::to_string(kCellsPerBlock) + " cells)");
+                                    " are supported");
   if (!diag || !ax || !ay || !az || !f || !p) return fail_na(CAMS_EINVAL, "null input pointer");
   if (!r && !norm_out) return fail_na(CAMS_EINVAL, "no output requested");
   int dev = 0;
@@ -197,7 +193,7 @@ extern "C" int cams_residual_norm_noalloc(int nx, int ny, int nz, const double* 
   // earlier call's error, still pending in the runtime, is not this one's.
   double s2 = 0.0;
   const bool direct = norm_out && cams::host_writable(dev);
-  double* total = direct ? &s2 : scratch + kMaxBlocks;
+  double* total = direct ? &s2 : scratch + cams::kColBlocks;
   const char* what = "launch: ";
   cams::ColWork w = cams::col_work(g, kSmallThreads);
   if (w.pieces <= (unsigned)kSmallPieces && small_fits(dev)) {

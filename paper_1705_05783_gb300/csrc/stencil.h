@@ -18,7 +18,9 @@
 namespace cams {
 
 constexpr int kColThreads = 256;    // threads of a CTA, one column each
-constexpr int kColBlocks = 6 * 152; // CTAs: six on each SM, one wave
+// CTAs of a launch at most: six for each of the 152 SMs (the residual's 64
+// registers a thread leave four of them resident at once, the assembly's 80 three).
+constexpr int kColBlocks = 6 * 152;
 
 // A launch's work: pieces of `threads` columns x `planes` planes.
 struct ColWork {
