@@ -289,8 +289,9 @@ __device__ __forceinline__ typename Word<T>::U wait_bits(const T* p, int* abort_
 // path, so they go ahead of the copies) and stages the operands of the group
 // kG - 1 ahead; values still unset are re-polled together; the kU steps
 // themselves are straight-line code.  Returns false after an abort or a
-// timeout (the warp's copies drained).
-template <class Op>
+// timeout (the warp's copies drained).  kOwnEnd: the end of the tile's copies
+// takes a path of its own (own_end; the arithmetic is the same).
+template <class Op, bool kOwnEnd>
 __device__ __forceinline__ bool factor_tile(const Geo& g, const Skew& sk, const Op& op,
                                             const typename Op::Scalar* out, int* abort_flag,
                                             int* status, typename Op::Scalar* ringw, int lane,
@@ -313,20 +314,20 @@ __device__ __forceinline__ bool factor_tile(const Geo& g, const Skew& sk, const 
   // Operands of steps gs .. gs+kU-1 into ring slot q, laid out
   // [slot][operand][step][lane], clamped to my row (read, then discarded).
   T* const ring = ringw + lane;
-  // (The end of the tile on a path of its own: with one commit for both cases an
-  // FP32 step takes 8% longer, 23.9 against 22.2 ms for a row of 10^5 cells.)
   auto stage = [&](int gs, int q) {
-    if (gs >= sk.ns) {
+    if (kOwnEnd && gs >= sk.ns) {
       cp_async_commit();
       return;
     }
+    if (kOwnEnd || gs < sk.ns) {
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      long long i = i0 + (gs + u);
-      i = i < row ? row : i;
-      i = i > row + g.nx - 1 ? row + g.nx - 1 : i;
+      for (int u = 0; u < kU; ++u) {
+        long long i = i0 + (gs + u);
+        i = i < row ? row : i;
+        i = i > row + g.nx - 1 ? row + g.nx - 1 : i;
 #pragma unroll
-      for (int a = 0; a < kN; ++a) cp_async(ring + ((q * kN + a) * kU + u) * kR, op.src(a, i));
+        for (int a = 0; a < kN; ++a) cp_async(ring + ((q * kN + a) * kU + u) * kR, op.src(a, i));
+      }
     }
     cp_async_commit();
   };
@@ -449,7 +450,7 @@ constexpr int ring_bytes() {
 // ctrl: [0] ticket, [1] abort flag.  `out` is the vector the operator
 // publishes into (pre-filled with the sentinel on every cell).  Each warp
 // claims tiles on its own.
-template <class Op>
+template <class Op, bool kOwnEnd>
 __global__ void __launch_bounds__(32 * kWarps, 1) k_factor(Geo g, Skew sk, Op op,
                                                             const typename Op::Scalar* out,
                                                             int* ctrl, int* status) {
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_factor(Geo g, Skew sk, Op op
     if (t >= ntiles) return;
     int Y, Z;
     tile_of_ticket(t, sk.nty, sk.ntz, Y, Z);
-    if (!factor_tile<Op>(g, sk, op, out, ctrl + 1, status, ringw, lane, Y, Z)) return;
+    if (!factor_tile<Op, kOwnEnd>(g, sk, op, out, ctrl + 1, status, ringw, lane, Y, Z)) return;
   }
 }
 
@@ -504,6 +505,18 @@ IluSet<float> set_of(Buffers& b, float*) {
   return IluSet<float>{f.Ad, f.Ax, f.Ay, f.Az, f.Axu, f.Ayu, f.Azu, f.Qx, f.Qy, f.Qz, f.dinv};
 }
 
+// Which of the two forms of a tile's copies (the compiler schedules the step
+// differently): with one commit for both cases an FP32 step takes 8% longer where a
+// tile has an SM's issue slots nearly to itself (a row of 10^5 cells 23.9 against
+// 22.2 ms, 4 x 4 x 16384 11.6 against 10.6, 1000 x 1000 839 against 803 us), and 1
+// to 8% less where many tiles of both directions run (200 x 200 x 100 496 against
+// 537 us, 128^3 323 against 334; 64^3, 8 tiles wide, 139.4 against 138.6).  FP64
+// takes up to 2% less with a path of its own everywhere.
+template <class T>
+bool own_end(const Skew& sk) {
+  return sizeof(T) == 8 || sk.nty <= 8 || sk.ntz <= 8;
+}
+
 // The pivot wavefront (level-scheduled or pipelined); returns the launch count.
 template <class Op>
 int factor_sweep(const Geo& g, Buffers& b, bool pipelined, int sms, const Op& fa,
@@ -522,7 +535,8 @@ int factor_sweep(const Geo& g, Buffers& b, bool pipelined, int sms, const Op& fa
   e = cudaMemsetAsync(ctrl, 0, 4 * sizeof(int), s);
   if (e != cudaSuccess) return 1;
   const int ctas = (sk.nty * sk.ntz + kWarps - 1) / kWarps;
-  k_factor<Op><<<ctas < sms ? ctas : sms, 32 * kWarps, ring_bytes<Op>(), s>>>(g, sk, fa, dinv, ctrl,
+  auto* kern = own_end<T>(sk) ? k_factor<Op, true> : k_factor<Op, false>;
+  kern<<<ctas < sms ? ctas : sms, 32 * kWarps, ring_bytes<Op>(), s>>>(g, sk, fa, dinv, ctrl,
                                                                              b.status);
   e = cudaGetLastError();
   return 2;
@@ -557,10 +571,13 @@ int ilu_ctrl_ints(const Geo& g) {
 }
 
 bool ilu_set_smem() {
-  return raise_smem_limit(k_factor<Factor<double>>, ring_bytes<Factor<double>>()) == cudaSuccess &&
-         raise_smem_limit(k_factor<Factor<float>>, ring_bytes<Factor<float>>()) == cudaSuccess &&
-         raise_smem_limit(k_factor<Factor<double, true>>, ring_bytes<Factor<double, true>>()) == cudaSuccess &&
-         raise_smem_limit(k_factor<Factor<float, true>>, ring_bytes<Factor<float, true>>()) == cudaSuccess;
+  auto allow = [](auto* kern, int bytes) { return raise_smem_limit(kern, bytes) == cudaSuccess; };
+  return allow(k_factor<Factor<double>, true>, ring_bytes<Factor<double>>()) &&
+         allow(k_factor<Factor<float>, true>, ring_bytes<Factor<float>>()) &&
+         allow(k_factor<Factor<float>, false>, ring_bytes<Factor<float>>()) &&
+         allow(k_factor<Factor<double, true>, true>, ring_bytes<Factor<double, true>>()) &&
+         allow(k_factor<Factor<float, true>, true>, ring_bytes<Factor<float, true>>()) &&
+         allow(k_factor<Factor<float, true>, false>, ring_bytes<Factor<float, true>>());
 }
 
 cudaError_t launch_ilu_factor(const Geo& g, Buffers& b, bool pipelined, int sms, bool single,
